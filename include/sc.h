@@ -303,9 +303,12 @@ sc_status sc_table_count(sc_ctx* ctx, const sc_mirror_t* mirror, const sc_incide
                          int* fp32_ok);
 
 /*
- * How the FP32 path cuts a request of n_omega uniform omegas into chunks, on
- * the host only (ctx may be NULL: planning on).  Each chunk is one pass of a
- * field kernel over the node tables.  The sizes minimise the summed field
+ * How the direct and grouped kernels of the FP32 path cut a request of n_omega
+ * uniform omegas into chunks, on the host only (ctx may be NULL: planning on).
+ * Each chunk is one pass of a field kernel over the node tables.  By default
+ * 25 and more omegas run on the tensor kernel instead, in chunks of up to 256,
+ * and this plan holds for fewer, for a rest below 25, and for everything when
+ * SC_OPT_TILE_LAYOUT is 0 or 1.  The sizes minimise the summed field
  * time of the chunks under field throughputs per omega count measured on
  * GB300, each extra chunk charged 2% of a 32-omega chunk: e.g. 65 omegas run
  * as 64 + 1 (on 16 threads of 8 omegas, 7 would idle), 33 as 1 + 32.
@@ -585,7 +588,8 @@ enum {
                                 /* they take the most splits whose workspace fits)  */
     SC_OPT_OMEGA_CHUNKS = 7,    /* 1 (default): cut a request's omegas into chunks  */
                                 /* that keep the field kernels' threads busy;      */
-                                /* 0: one chunk per 2048 omegas                     */
+                                /* 0: one chunk per 2048 omegas, on the direct and  */
+                                /* grouped kernels                                  */
     SC_OPT_MFIE_ORDER = 9,      /* 0 (default): physical optics; 1: add the first  */
                                 /* correction of the MFIE's Liouville-Neumann      */
                                 /* series (see below; sc_eval, sc_eval_time_domain) */
@@ -597,10 +601,12 @@ enum {
     SC_OPT_TILE_LAYOUT = 13,    /* tile shape of the FP32 field kernel (threads per */
                                 /* point x omegas per thread) for chunks of 8,      */
                                 /* 9..16, 33..64 and 65..128 omegas, which have two */
-                                /* near layouts: -1 (default) the autotuner times   */
+                                /* near layouts: -1 (default) the tensor kernel from */
+                                /* 25 omegas on and below that the autotuner times  */
                                 /* both on the first chunk of each shape when       */
                                 /* SC_OPT_AUTOTUNE is on (else the default); 0 the  */
-                                /* default layout; 1 the alternative.  Other omega  */
+                                /* default layout; 1 the alternative, both without  */
+                                /* the tensor kernel.  Other omega                  */
                                 /* counts have one layout.  sc_eval_stats reports   */
                                 /* the layout taken                                 */
     SC_OPT_SERVE_PRIORITY = 14, /* 1 (default): serving runs short requests first   */

@@ -762,6 +762,9 @@ sc_status sc_eval_fp32_static(sc_ctx* ctx, const sc_mirror_t* m, const sc_incide
     f.nodes = tab->d32;
     f.n_surf_tiles = tab->n_surf_tiles;
     f.n_rim_tiles = tab->n_rim_tiles;
+    f.amax_surf = tab->parts[0].amax_surf;
+    f.amax_rim = tab->parts[0].amax_rim;
+    f.pmin = tab->pmin;
     f.tiles_per_split = tab->n_surf_tiles;  // one surface split and the rim slot
     f.n_splits = 1;
     f.flush_tiles = (int)std::max<long long>(1, ctx->flush_nodes / sc::kTile);

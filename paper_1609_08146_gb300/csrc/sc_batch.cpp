@@ -138,6 +138,10 @@ sc_status choose_splits(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int s
     return SC_OK;
 }
 
+// The tensor kernel is on unless the caller pins the FP32 kernels' chunks or
+// tile shapes.
+bool tensor_on(const sc_ctx* ctx) { return ctx->omega_chunks && ctx->tile_layout == -1; }
+
 // Kernel class (tile shape: threads per point x omegas per thread) of a
 // chunk.  field_class(n) is the layout measured fastest on GB300 for n
 // omegas; where a second layout of the same n is close (alt_field_class), the
@@ -149,6 +153,11 @@ sc_status choose_class(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int* c
 {
     const int def = sc::field_class(c.f.n_omega);
     *cls_out = def;
+    const int ten = sc::tensor_class(c.f.n_omega);
+    if (ten >= 0 && tensor_on(ctx)) {
+        *cls_out = ten;
+        return SC_OK;
+    }
     const int alt = sc::alt_field_class(c.f.n_omega);
     if (alt < 0 || ctx->tile_layout == 0) return SC_OK;
     if (ctx->tile_layout == 1) {
@@ -304,6 +313,10 @@ sc_status plan_request(sc_ctx* ctx, Lane& ln, const Table* tab, const double* om
     const bool small_cuts = (long long)n_points * tab->n_surf >= kSmallCutPairs;
     for (int o0 = 0, no = 0; o0 < n_omega; o0 += no) {
         no = ctx->omega_chunks ? next_chunk(n_omega - o0, small_cuts) : std::min(kMaxChunk, n_omega - o0);
+        // the tensor kernel takes its counts whole: a pair costs it nearly the
+        // same whatever the count, so no cut pays
+        const bool ten = tensor_on(ctx) && n_omega - o0 >= sc::kTensorMinOmega;
+        if (ten) no = std::min(sc::kTensorMaxOmega, n_omega - o0);
         Chunk c;
         const double w0 = omegas[o0];
         c.f.nodes = tab->d32;
@@ -400,6 +413,10 @@ sc_status launch_chunks(sc_ctx* ctx, Lane& ln, std::vector<Chunk>& ch, float2* w
             w.f = c.f;
             w.f.nodes = c.tab->parts[t].d32;
             w.f.n_rim_tiles = c.tab->parts[t].n_rim_tiles;
+            w.f.amax_surf = c.tab->parts[t].amax_surf;
+            w.f.amax_rim = c.tab->parts[t].amax_rim;
+            w.f.pmin = c.tab->pmin;
+            if (sc::is_tensor_class(c.cls)) sc::tensor_prepare(c.cls, w.f);
             w.f.ws = c.f.ws + (size_t)t * (c.ws_elems / c.n_parts);
             w.pb = c.pb;
             w.cls = c.cls;

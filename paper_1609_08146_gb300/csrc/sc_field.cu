@@ -1,6 +1,7 @@
 // sc_field.cu -- FP32 field-sum kernels of libsc (the hot path): the grouped
 // kernel and the class dispatch; the direct kernel of requests with few
-// omegas is in sc_field_direct.cu, their shared device helpers in
+// omegas is in sc_field_direct.cu, the tensor-core kernel that takes 25 to 256
+// omegas by default in sc_field_tensor.cu, their shared device helpers in
 // sc_field_common.cuh.
 //
 // Computes, for every observation point r' and frequency omega_n, the
@@ -398,7 +399,8 @@ void class_layout(int cls, int* tpp, int* opt)
         {2, 5}, {2, 6}, {2, 7}, {2, 8}, {4, 5}, {4, 6}, {4, 8},             // 8..14
         {8, 5}, {8, 6}, {8, 7}, {8, 8}, {16, 8}, {32, 8},                   // 15..20
         {64, 8}, {128, 8}, {256, 8},                                        // 21..23 grouped
-        {1, 8}, {4, 3}, {4, 4}, {16, 3}, {16, 4}, {32, 4}};                 // 24..29
+        {1, 8}, {4, 3}, {4, 4}, {16, 3}, {16, 4}, {32, 4},                  // 24..29
+        {64, 2}, {64, 4}};                                                  // 30, 31 tensor (rows)
     const int c = cls < 0 || cls >= kNumClasses ? 0 : cls;
     *tpp = kLayout[c][0];
     *opt = kLayout[c][1];
@@ -407,6 +409,7 @@ void class_layout(int cls, int* tpp, int* opt)
 void field_shape(int cls, int device, int* ppc, int* slots)
 {
     if (is_direct_class(cls)) return direct_field_shape(cls, device, ppc, slots);
+    if (is_tensor_class(cls)) return tensor_field_shape(cls, device, ppc, slots);
     switch (cls) {
     case 21: return grouped_shape<64>(device, ppc, slots);
     case 22: return grouped_shape<128>(device, ppc, slots);
@@ -418,6 +421,7 @@ int launch_field_batch(int cls, const BatchLaunch& b, int grid, cudaStream_t s)
 {
     if (grid < 1) return 0;
     if (is_direct_class(cls)) return launch_direct_field(cls, b, grid, s);
+    if (is_tensor_class(cls)) return launch_tensor_field(cls, b, grid, s);
     switch (cls) {
     case 21: return launch_grouped<64>(b, grid, s);
     case 22: return launch_grouped<128>(b, grid, s);
@@ -428,7 +432,8 @@ int launch_field_batch(int cls, const BatchLaunch& b, int grid, cudaStream_t s)
 
 int launch_field_f32(const FieldLaunch& p, cudaStream_t s)
 {
-    const int cls = field_class(p.n_omega);
+    const int ten = tensor_class(p.n_omega);
+    const int cls = ten >= 0 ? ten : field_class(p.n_omega);
     int ppc = 1, slots = 1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -436,6 +441,7 @@ int launch_field_f32(const FieldLaunch& p, cudaStream_t s)
     BatchLaunch b{};
     b.reqs = nullptr;
     b.one.f = p;
+    if (ten >= 0) tensor_prepare(ten, b.one.f);
     b.one.pb = (p.n_pts + ppc - 1) / ppc;
     b.one.cls = cls;
     b.one.item0 = 0;
@@ -445,7 +451,7 @@ int launch_field_f32(const FieldLaunch& p, cudaStream_t s)
     b.err = p.err;
     b.abort = nullptr;  // grid mode: one item per CTA, nothing to stop early
     b.fail_tile = -1;
-    return launch_field_batch(cls, b, (int)b.n_items, s);
+    return launch_field_batch(cls, b, (int)(ten >= 0 ? std::min<long long>(slots, b.n_items) : b.n_items), s);
 }
 
 namespace {

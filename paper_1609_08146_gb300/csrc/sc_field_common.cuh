@@ -3,7 +3,8 @@
 // the direct kernel, few): mbarrier and bulk-copy wrappers with bounded
 // waits, the reduced phasor e^{i pi x}, the pair geometry and coefficients of
 // Eq. 11's summand, the packed accumulation step, the compensated fold, and
-// the persistent work-item loop.  Included by those two files only.
+// the persistent work-item loop.  Included by those two files and the tensor
+// kernel (sc_field_tensor.cu) only.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -334,8 +335,14 @@ __device__ __forceinline__ Item decode(const BatchLaunch& b, long long item)
     Item it;
     it.r = find_req(b, item);
     const long long local = item - it.r->item0;
-    it.pbi = (int)(local % it.r->pb);
-    it.split = (int)(local / it.r->pb);
+    if (local >> 32) {
+        it.pbi = (int)(local % it.r->pb);
+        it.split = (int)(local / it.r->pb);
+    } else {  // a 64-bit division costs over a hundred instructions
+        const unsigned l = (unsigned)local, pb = (unsigned)it.r->pb;
+        it.split = (int)(l / pb);
+        it.pbi = (int)(l - (unsigned)it.split * pb);
+    }
     return it;
 }
 

@@ -1,0 +1,829 @@
+// sc_field_tensor.cu -- the FP32 field sum as a contraction on the tensor
+// cores (tcgen05), for chunks of a few dozen to 256 omegas.  The quadrature of
+// Sec. II, Eq. 11 over the node table with the compensated phase of
+// Sec. III.C.1; see sc_field.cu for the summand.
+//
+// For one point the sums over the nodes j are S_c(omega) = sum_j C_cj e^{i k
+// Phi_j} with twelve real coefficients per pair,
+//     C = (U + V, Wv, V/R, Wv/R),  E = ik S_{U+V} - S_{V/R},  B = ik S_W - S_{W/R}.
+// On the uniform grid omega = Omega_{n1} + delta_{n2} the phase factor is a
+// product of a row phasor e^{i 2 pi Omega_{n1} Phi} and a column phase
+// theta_{n2} = 2 pi delta_{n2} Phi, with the offsets delta symmetric about
+// zero, so that +delta and -delta share their cosine and sine columns:
+//     D[row, col] = sum_j A[row, j] B[col, j]
+//   rows  64 row phasors, cosine and sine (M = 128),
+//   cols  12 coefficients times N2 trigonometric columns (N = 12 N2),
+//   K     the nodes.
+// N2 omegas per row phasor come out of 12 N2 real columns: no product is
+// computed twice, and a pair costs 128 + 12 N2 operand values instead of the
+// direct kernel's 24 FP32 operations for each of its 64 N2 omegas.
+//
+// Precision.  Every operand value x is split into two halves, hi = fp16(x) and
+// lo = fp16(x - hi), 22 bits in all, and three products are accumulated: hi hi
+// in one set of TMEM columns, hi lo + lo hi in another.  What is dropped (lo
+// lo and the rounding of lo) is below 2^-23 of the largest operand, the size
+// of one FP32 rounding.  The coefficients are brought into the range of fp16
+// by powers of two chosen per point from bounds on the table's largest source
+// and the smallest distance.  The tensor cores' accumulation drops the bits
+// below the accumulator's last place instead of rounding, which makes coherent
+// sums too small, by half a last place per MMA (measured: 1.2e-7 per node
+// tile).  So a run of accumulation is only kFoldTiles tiles (160 nodes; the
+// direct kernel's FP32 runs have 2048), the expected loss, one last place per
+// tile after the first, is given back when the run is read, and the runs are
+// summed outside the tensor cores by Kahan's rule.  Against FP64, relative
+// norms over sizes and beams at random: 1.9e-7 to 4.1e-7 here, 2.8e-7 to
+// 1.1e-6 with the FP32 kernels.
+//
+// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 63 ms, 4.4e12
+// evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
+// Shared memory is busy 72% of the time, half by the operands' stores and half
+// by the MMAs' reads of them, the schedulers issue in 60% of the cycles, and
+// the tensor pipe works 26%.  A pair's cost is mostly its 128 row values and
+// depends little on N2, so the rate falls in proportion to the omega count:
+// 2.95e12 at 128 omegas, 1.6e12 at 48, 1.1e12 at 32 (direct: 1.14, 1.04,
+// 1.00e12); the lines between the classes lie where the measured rates cross:
+// from 25 omegas the tensor kernel (24: direct 0.98, tensor 0.85e12; 26: 0.83,
+// 0.91), 4 omegas per row phasor above 128.
+//
+// Structure (one CTA per SM, 16 warps; shared memory holds ten stages):
+//   warps 0-3   read a finished accumulator (TMEM, two of them), keep the
+//               compensated running sums of the item (one point, one node
+//               split) in registers and write its partials;
+//   warps 4, 8  issue the MMAs, one warp for either accumulator;
+//   the others  produce operands, each into a stage of its own: lane = node,
+//               five warps per accumulator.  A lane computes its pair's
+//               geometry, coefficients and phases and writes its operand
+//               columns in the MN-major core-matrix layout (8 rows of one node
+//               are 16 contiguous bytes, so that a warp's stores are
+//               conflict-free); no data passes between lanes.
+// Items are strided over the CTAs (item = blockIdx + i gridDim), which every
+// role follows on its own; all waits are bounded as in the other kernels.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "sc_field_common.cuh"
+#include "sc_internal.h"
+
+namespace sc {
+
+namespace {
+
+constexpr int kRows = 64;                   // row phasors (cosine and sine: M = 128)
+constexpr int kFoldTiles = 5;               // node tiles per run of an accumulator
+constexpr int kStages = 2 * kFoldTiles;     // operand stages (one node tile each): half for either accumulator
+constexpr int kProd = kStages;              // producer warps, each with a stage of its own
+constexpr int kTensorThreads = 512;
+static_assert(4 + 2 + kProd <= kTensorThreads / 32, "warps");
+// Registers: 128 a thread at launch; the epilogue's warpgroup takes 176 and
+// the other three 112 (128 * 176 + 384 * 112 = 65536).
+constexpr int kEpiRegs = 176, kOtherRegs = 112;
+static_assert(128 * kEpiRegs + 384 * kOtherRegs <= 65536, "register split");
+constexpr int kBlkBytes = kTile * 16;           // a block of 8 rows (or columns) of a stage's 32 nodes
+constexpr int kABytes = 2 * kRows / 8 * kBlkBytes;  // one half (hi or lo) of A
+
+template <int N2>
+struct Tens {
+    static constexpr int N = 12 * N2;
+    static constexpr int NP = (N + 7) / 8 * 8;     // rounded to core matrices
+    static constexpr int NC = (NP + 15) / 16 * 16; // the lo x hi product's columns (M = 128 wants 16s)
+    static constexpr int DCOLS = NP + NC;          // one accumulator: NP hi hi, then hi lo + lo hi
+    static constexpr int ALLOC = DCOLS <= 32 ? 64 : (DCOLS <= 64 ? 128 : (DCOLS <= 128 ? 256 : 512));
+    static constexpr int STAGE = 2 * kABytes + 2 * (NP / 8) * kBlkBytes;
+    static constexpr int OFF_BAR = kStages * STAGE;
+    static constexpr int SMEM = OFF_BAR + 256;
+    static_assert(2 * NP % 16 == 0, "hi product width");
+    static_assert(2 * DCOLS <= ALLOC, "tensor memory");
+    static_assert(SMEM <= 227 * 1024, "shared memory");
+};
+
+// ------------------------------------------------------------------------
+// tcgen05 wrappers
+
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
+{
+    // no swizzle, MN-major: core matrices of 8 MN x 8 K; 128 bytes from one
+    // block of 8 K to the next (leading offset), kBlkBytes from one block of 8
+    // MN to the next (stride offset)
+    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(kBlkBytes >> 4) << 32) |
+           (1ull << 46);
+}
+
+// f16 x f16 -> f32, A and B MN-major, M = 128
+__host__ __device__ constexpr uint32_t mma_idesc(int n)
+{
+    return (1u << 4) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(2 * kRows >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_commit(uint64_t* bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                 : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t v[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// One look at an mbarrier's phase, without waiting.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// ------------------------------------------------------------------------
+// Operand splitting: eight FP32 values -> eight fp16 (16 bytes) of the high
+// parts and eight of the low parts.
+
+__device__ __forceinline__ uint32_t pack_h2(float a, float b)
+{
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+__device__ __forceinline__ void split_store8(unsigned char* hi, unsigned char* lo, const float2 x[4])
+{
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        h[i] = pack_h2(x[i].x, x[i].y);
+        float rx, ry;  // x - hi, exact (one mixed-precision FMA each)
+        asm("{\n\t.reg .b16 a, b, m;\n\tmov.b32 {a, b}, %2;\n\tmov.b16 m, 0xBC00;\n\t"
+            "fma.rn.f32.f16 %0, a, m, %3;\n\tfma.rn.f32.f16 %1, b, m, %4;\n\t}"
+            : "=f"(rx), "=f"(ry)
+            : "r"(h[i]), "f"(x[i].x), "f"(x[i].y));
+        l[i] = pack_h2(rx, ry);
+    }
+    *reinterpret_cast<uint4*>(hi) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(lo) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Segments of eight row phasors that n_omega omegas take, and the one the
+// seeds start from (then outwards both ways).
+__host__ __device__ inline int segments(int n_omega, int n2) { return ((n_omega + n2 - 1) / n2 + 7) / 8; }
+__host__ __device__ inline int seed_seg(int nseg) { return nseg >> 1; }
+
+// ------------------------------------------------------------------------
+// One work item as every role sees it.
+
+struct TItem {
+    const FieldLaunch* f;
+    int pt, split, t0, nt;
+    float4 P;        // point and |r'|^2
+    float js, rs;    // powers of two: sources times js, 1/R times rs
+    bool ok;         // operands fit fp16 (see below); otherwise the item takes the plain FP32 loop
+};
+
+__device__ __forceinline__ TItem tensor_item(const BatchLaunch& b, long long item)
+{
+    const Item w = decode(b, item);
+    TItem t;
+    t.f = &w.r->f;
+    t.pt = w.pbi;
+    t.split = w.split;
+    int t1;
+    split_range(*t.f, w.split, t.t0, t1);
+    t.nt = t1 - t.t0;
+    load_point(t.f->pts, t.f->n_pts, w.pbi, t.P);  // (|r'|^2 dropped by the roles that do not use it)
+    // R >= |P| - |r'| >= rmin on every node; |J|, |rho| <= amax.  The powers of
+    // two bring |U + V|, |Wv| below 2^12 and 1/R below 1.  Points within 1/16
+    // of the mirror's smallest distance (or sources out of range, or NaN) do
+    // not qualify: their 1/R spans too much for one scale.
+    const float amax = w.split < t.f->n_splits ? t.f->amax_surf : t.f->amax_rim;
+    const float rmin = t.f->pmin - sqrtf(fmaf(t.P.x, t.P.x, fmaf(t.P.y, t.P.y, t.P.z * t.P.z)));
+    t.ok = rmin >= 0.0625f * t.f->pmin && rmin > 1e-30f && rmin < 1e30f && amax < 1e30f && amax >= 0.f;
+    t.js = t.rs = 1.f;
+    if (t.ok) {
+        t.rs = ldexpf(1.f, ilogbf(rmin));
+        if (amax > 0.f) {
+            const int e = 10 - ilogbf(amax / rmin);
+            t.ok = e > -100 && e < 100;
+            t.js = t.ok ? ldexpf(1.f, e) : 1.f;
+        }
+    }
+    return t;
+}
+
+// The launch's abort word, read between items by the MMA warps, which pass it
+// on to their CTA's word; every wait of the other roles ends on that.
+__device__ __forceinline__ bool launch_aborted(const BatchLaunch& b, volatile int* s_abort)
+{
+    if (b.abort && *(const volatile int*)b.abort) *s_abort = 1;
+    return *s_abort != 0;
+}
+
+// ------------------------------------------------------------------------
+// Producers
+
+// One segment: eight row phasors from the seed of its fourth, its neighbour by
+// one rotation, and the three-term recurrence from these two outwards: three
+// steps at most, so that the rounding of c = 2 cos, which n steps multiply by
+// n (n + 1) / 2, is multiplied by 6 and not by the 21 of a chain from one end.
+// Steps alternate -c, -c, +c, which saves the negation; slots 1, 2, 5, 6 come
+// out negated and the epilogue turns them back.
+__device__ __forceinline__ void store_segment(unsigned char* a_hi, float2 seed, float2 rot, float2 cc, float2 ncc)
+{
+    float2 ph[8];
+    ph[3] = seed;
+    ph[4] = cmul(seed, rot);
+#pragma unroll
+    for (int j = 1; j < 4; ++j) {
+        ph[4 + j] = __ffma2_rn((j & 1) ? ncc : cc, ph[3 + j], ph[2 + j]);
+        ph[3 - j] = __ffma2_rn((j & 1) ? ncc : cc, ph[4 - j], ph[5 - j]);
+    }
+    const float2 c[4] = {make_float2(ph[0].x, ph[1].x), make_float2(ph[2].x, ph[3].x),
+                         make_float2(ph[4].x, ph[5].x), make_float2(ph[6].x, ph[7].x)};
+    const float2 d[4] = {make_float2(ph[0].y, ph[1].y), make_float2(ph[2].y, ph[3].y),
+                         make_float2(ph[4].y, ph[5].y), make_float2(ph[6].y, ph[7].y)};
+    split_store8(a_hi, a_hi + kABytes, c);
+    split_store8(a_hi + kBlkBytes, a_hi + kABytes + kBlkBytes, d);
+}
+
+// One tile's operands; `wait` (bounded) blocks until the MMAs have read the
+// stage's last contents and is placed after everything that can be computed
+// without the stage.  False: aborted or expired.
+template <int N2, typename Wait>
+__device__ __forceinline__ bool produce_tile(unsigned char* stage, const float nd[9], const TItem& it, int lane,
+                                             int nseg, const TensorSteps& w, Wait wait)
+{
+    using L = Tens<N2>;
+    const float px = nd[0], py = nd[1], pz = nd[2], pn = nd[3], wo = nd[4];
+    const float4 P = it.P;
+    // pair geometry and phase as in pair_coefs()
+    const float dx = px - P.x, dy = py - P.y, dz = pz - P.z;
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float ir = rsqrtf(r2);
+    const float R = r2 * ir;
+    const float D = fmaf(-2.0f * P.x, px, fmaf(-2.0f * P.y, py, fmaf(-2.0f * P.z, pz, P.w)));
+    const float phi = __fdividef(D, R + pn) + wo;
+    const float rx = dx * ir, ry = dy * ir, rz = dz * ir;
+    const float sir = it.js * ir;
+    const float ux = nd[5] * sir, uy = nd[6] * sir, uz = nd[7] * sir;
+    const float a = nd[8] * sir;
+    const float irs = ir * it.rs;
+    float co[12];
+    const float vx = a * rx, vy = a * ry, vz = a * rz;
+    co[0] = ux + vx; co[1] = uy + vy; co[2] = uz + vz;
+    co[3] = fmaf(uy, rz, -uz * ry);
+    co[4] = fmaf(uz, rx, -ux * rz);
+    co[5] = fmaf(ux, ry, -uy * rx);
+    co[6] = vx * irs; co[7] = vy * irs; co[8] = vz * irs;
+    co[9] = co[3] * irs; co[10] = co[4] * irs; co[11] = co[5] * irs;
+
+    // cosines and sines of the column offsets: m steps (odd N2) or m + 1/2 (even)
+    float trig[N2];
+    {
+        float2 q = N2 > 1 ? phasor_2wphi(w.col.x, w.col.y, phi) : make_float2(1.f, 0.f);
+        const float2 full = (N2 & 1) ? q : cmul(q, q);
+        if (N2 & 1) trig[0] = 1.f;
+#pragma unroll
+        for (int m = 0; m < N2 / 2; ++m) {
+            trig[(N2 & 1) + 2 * m] = q.x;
+            trig[(N2 & 1) + 2 * m + 1] = q.y;
+            if (m + 1 < N2 / 2) q = cmul(q, full);
+        }
+    }
+    // row phasors: one seed (MUFU sine and cosine, as in the direct kernel) and
+    // the rotations between rows and between segments
+    const float2 rot = phasor_2wphi(w.row.x, w.row.y, phi);
+    const float2 rseg = phasor_2wphi(w.seg.x, w.seg.y, phi);
+    float2 up = phasor_2wphi_mufu(w.seed.x, w.seed.y, phi);
+    if (!wait()) return false;
+
+    unsigned char* b_hi = stage + 2 * kABytes + lane * 16;
+    unsigned char* b_lo = b_hi + (L::NP / 8) * kBlkBytes;
+#pragma unroll
+    for (int blk = 0; blk < L::NP / 8; ++blk) {
+        float2 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c0 = blk * 8 + 2 * i;
+            v[i].x = c0 < L::N ? co[c0 % 12] * trig[c0 < L::N ? c0 / 12 : 0] : 0.f;
+            v[i].y = c0 + 1 < L::N ? co[(c0 + 1) % 12] * trig[c0 + 1 < L::N ? (c0 + 1) / 12 : 0] : 0.f;
+        }
+        split_store8(b_hi + blk * kBlkBytes, b_lo + blk * kBlkBytes, v);
+    }
+    // segments outwards from the seed's, two independent chains
+    const float2 cc = make_float2(2.f * rot.x, 2.f * rot.x);
+    const float2 ncc = make_float2(-cc.x, -cc.y);
+    const float2 rback = make_float2(rseg.x, -rseg.y);
+    float2 dn = cmul(up, rback);
+    const int s0 = seed_seg(nseg);
+    unsigned char* a_up = stage + lane * 16 + 2 * s0 * kBlkBytes;
+    unsigned char* a_dn = a_up - 2 * kBlkBytes;
+    store_segment(a_up, up, rot, cc, ncc);
+    const int both = nseg - 1 - s0;  // segments on either side (an even count has one more below)
+#pragma unroll 1
+    for (int s = 0; s < both; ++s) {
+        up = cmul(up, rseg);
+        a_up += 2 * kBlkBytes;
+        store_segment(a_dn, dn, rot, cc, ncc);
+        store_segment(a_up, up, rot, cc, ncc);
+        a_dn -= 2 * kBlkBytes;
+        dn = cmul(dn, rback);
+    }
+    if (s0 > both) store_segment(a_dn, dn, rot, cc, ncc);
+    return true;
+}
+
+__device__ __forceinline__ void load_node(const FieldLaunch& p, int tile, int lane, float nd[9])
+{
+    const float* src = p.nodes + (size_t)tile * kTileFloats + lane;
+#pragma unroll
+    for (int f = 0; f < 9; ++f) nd[f] = __ldg(src + f * kTile);
+}
+
+// ------------------------------------------------------------------------
+// Epilogue
+
+__device__ __forceinline__ void two_sum(float& s, float& e, float v)
+{
+    const float t = s + v, b = t - s;
+    e += (s - (t - b)) + (v - b);
+    s = t;
+}
+
+// The item's partials from the running sums s - e of the lane's row.  With CC,
+// CS the cosine row's sums over the cosine and sine columns of an offset
+// phi > 0, and SC, SS the sine row's, the sums at +-phi are
+//     Re = CC -+ SS,   Im = SC +- CS,
+// and E = ik S1 - S2, B likewise (S1 over U + V or Wv, S2 over V/R or Wv/R).  A
+// cosine row (lane) writes real parts, Re E = -k Im S1 - Re S2, its partner (lane
+// ^ 8) imaginary ones, Im E = k Re S1 - Im S2: either needs the partner's cosine
+// column of S1 and sine column of S2, one exchange each.
+template <int N2>
+__device__ __forceinline__ void write_item(const TItem& it, int row, const float2* s2, const float2* e2)
+{
+    const FieldLaunch& p = *it.f;
+    const int seg = row >> 4, idx = row & 7;
+    const bool im = (row & 8) != 0;
+    const int n1 = seg * 8 + idx;
+    const float sg = ((idx + 1) & 2) ? -1.f : 1.f;
+    const float inv = sg / it.js, inv2 = 1.0f / it.rs;
+    auto s = [&](int c) { return (c & 1) ? s2[c >> 1].y : s2[c >> 1].x; };
+    auto e = [&](int c) { return -((c & 1) ? e2[c >> 1].y : e2[c >> 1].x); };
+    float2* base = p.ws + (((size_t)it.split * p.n_pts + it.pt) * (size_t)p.n_omega) * kAcc + (im ? 1 : 0);
+    constexpr int kOff = (N2 + 1) / 2;  // offsets: pairs +-phi, and zero if N2 is odd
+#pragma unroll
+    for (int o = 0; o < kOff; ++o) {
+        const bool zero = (N2 & 1) && o == 0;
+        const int tc = zero ? 0 : ((N2 & 1) ? 2 * o - 1 : 2 * o);  // its cosine column
+        float2 dst_v[2][6];
+        float k_h[2], k_l[2];
+        int nn[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // h = 0: +phi, 1: -phi
+            const int twice = zero ? 0 : (h == 0 ? 1 : -1) * ((N2 & 1) ? 2 * o : 2 * o + 1);
+            nn[h] = n1 * N2 + (twice + N2 - 1) / 2;
+            // k_n = k_0 + n dk as a float-float pair, with the sign of ik's product
+            const float fn = (float)nn[h], a = fn * p.steps.dk.x;
+            float kh = p.steps.k0.x, kl = fmaf(fn, p.steps.dk.x, -a) + fmaf(fn, p.steps.dk.y, p.steps.k0.y);
+            two_sum(kh, kl, a);
+            k_h[h] = im ? kh : -kh;
+            k_l[h] = im ? kl : -kl;
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const int c1 = tc * 12 + c, c2 = c1 + 6;
+            // partner's cosine column of S1 and sine (at zero offset: no) column of S2
+            const float p1 = __shfl_xor_sync(0xffffffffu, s(c1), 8), p1e = __shfl_xor_sync(0xffffffffu, e(c1), 8);
+            const float p2 = zero ? 0.f : __shfl_xor_sync(0xffffffffu, s(zero ? c2 : c2 + 12), 8);
+            const float p2e = zero ? 0.f : __shfl_xor_sync(0xffffffffu, e(zero ? c2 : c2 + 12), 8);
+            const float o1 = zero ? 0.f : s(zero ? c1 : c1 + 12), o1e = zero ? 0.f : e(zero ? c1 : c1 + 12);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (zero && h == 1) continue;
+                const float q1 = (im ? -1.f : 1.f) * (h == 0 ? 1.f : -1.f);  // S1: cosine rows +-, sine rows -+
+                const float q2 = -q1;                                       // S2: cosine rows -+, sine rows +-
+                float a = p1, al = fmaf(q1, o1e, p1e);
+                two_sum(a, al, q1 * o1);
+                float v = k_h[h] * a;
+                float vl = fmaf(k_h[h], a, -v) + fmaf(k_h[h], al, k_l[h] * a);
+                float r = s(c2), rl = fmaf(q2, p2e, e(c2));
+                two_sum(r, rl, q2 * p2);
+                two_sum(v, vl, -r * inv2);
+                dst_v[h][c] = make_float2(inv * v, inv * fmaf(-rl, inv2, vl));
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (!(zero && h == 1) && nn[h] < p.n_omega)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) base[(size_t)nn[h] * kAcc + 2 * c] = dst_v[h][c];
+    }
+}
+
+// ------------------------------------------------------------------------
+// Items whose operands do not fit fp16: the direct kernel's loop on the
+// producer warps.  Warp w sums every eighth node tile for all omegas (lane =
+// 8 consecutive omegas), sharing each tile's pair rows through its stage; every
+// flush the warps' sums are added, in warp order, to the compensated partials.
+
+// A bounded barrier of the producer warps (false: aborted or expired).
+struct ProdSync {
+    uint64_t* bar;
+    volatile int* s_abort;
+    int* launch_abort;
+    unsigned phase;
+    bool timed_out;
+    __device__ __forceinline__ bool sync(int lane)
+    {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+        return field_wait(bar, phase++ & 1, s_abort, launch_abort, timed_out) == WAIT_DONE;
+    }
+};
+
+template <int N2>
+__device__ __noinline__ bool plain_item(unsigned char* smem, const TItem& it, int w, int lane, ProdSync& ps)
+{
+    constexpr int NB = kRows * N2 / 32;  // omegas per lane
+    using L = Tens<N2>;
+    static_assert(L::STAGE >= kRows * N2 * 12 * 4 && L::STAGE >= 32 * 16 * 4, "stage too small for the plain loop");
+    const FieldLaunch& p = *it.f;
+    float* rows = reinterpret_cast<float*>(smem + w * L::STAGE);
+    const double om0 = (double)p.om_hi0 + (double)p.om_lo0, dom = (double)p.dom_hi + (double)p.dom_lo;
+    float kv[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) kv[j] = (float)(6.283185307179586 * (om0 + (double)(lane * NB + j) * dom));
+    const double wg = om0 + (double)(lane * NB) * dom;
+    const float wgh = (float)wg, wgl = (float)(wg - (double)wgh);
+    float2* dst = p.ws + ((size_t)it.split * p.n_pts + it.pt) * (size_t)p.n_omega * kAcc;
+    const int round = max(1, p.flush_tiles) * kProd;  // tiles per flush, all warps
+    for (int r0 = 0; r0 < it.nt || r0 == 0; r0 += round) {
+        AccX2 acc[NB];
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+#pragma unroll
+            for (int c = 0; c < kAcc / 2; ++c) acc[j].v[c] = make_float2(0.f, 0.f);
+        for (int t = r0 + w; t < min(it.nt, r0 + round); t += kProd) {
+            const float* nb = p.nodes + (size_t)(it.t0 + t) * kTileFloats;
+            float co[10];
+            const float phi = pair_coefs(nb, lane, it.P, co);
+            const float2 rot = phasor_2wphi(p.dom_hi, p.dom_lo, phi);
+            float4* r4 = reinterpret_cast<float4*>(rows + lane * 16);
+            r4[0] = make_float4(co[0], co[1], co[2], co[3]);
+            r4[1] = make_float4(co[4], co[5], co[6], co[7]);
+            r4[2] = make_float4(co[8], co[9], rot.x, rot.y);
+            r4[3] = make_float4(phi, 0.f, 0.f, 0.f);
+            __syncwarp();
+#pragma unroll 1
+            for (int q = 0; q < kTile; ++q) {
+                const float4* s4 = reinterpret_cast<const float4*>(rows + q * 16);
+                const float4 a0 = s4[0], a1 = s4[1], a2 = s4[2];
+                const float2 cp[10] = {make_float2(a0.x, a0.x), make_float2(a0.y, a0.y), make_float2(a0.z, a0.z),
+                                       make_float2(a0.w, a0.w), make_float2(a1.x, a1.x), make_float2(a1.y, a1.y),
+                                       make_float2(a1.z, a1.z), make_float2(a1.w, a1.w), make_float2(a2.x, a2.x),
+                                       make_float2(-a2.y, -a2.y)};
+                const float2 ro = make_float2(a2.z, a2.w);
+                const float2 cc = make_float2(2.f * ro.x, 2.f * ro.x), ncc = make_float2(-cc.x, -cc.x);
+                float2 p0 = phasor_2wphi_mufu(wgh, wgl, s4[3].x);
+                float2 p1 = cmul(p0, ro);
+                eval_x2<true>(acc[0], cp, kv[0], p0);
+                if (NB > 1) eval_x2<true>(acc[1], cp, kv[1], p1);
+#pragma unroll
+                for (int j = 2; j < NB; ++j) {
+                    const float2 pn = __ffma2_rn((j & 1) ? cc : ncc, p1, p0);
+                    eval_x2<true>(acc[j], cp, kv[j], pn);
+                    p0 = p1;
+                    p1 = pn;
+                }
+            }
+            __syncwarp();
+        }
+        // the warp's sums into its stage, then all warps' sums into the partials
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+#pragma unroll
+            for (int c = 0; c < kAcc / 2; ++c) {
+                const float sg = (j & 2) ? -1.f : 1.f;
+                float* r = rows + (lane * NB + j) * kAcc + 2 * c;
+                r[0] = sg * acc[j].v[c].x;
+                r[1] = sg * acc[j].v[c].y;
+            }
+        if (!ps.sync(lane)) return false;
+        for (int x = w * 32 + lane; x < p.n_omega * kAcc; x += 32 * kProd) {
+            float2 v = r0 == 0 ? make_float2(0.f, 0.f) : dst[x];
+            for (int u = 0; u < kProd; ++u)
+                two_sum(v.x, v.y, reinterpret_cast<const float*>(smem + u * L::STAGE)[x]);
+            dst[x] = v;
+        }
+        if (!ps.sync(lane)) return false;
+    }
+    return true;
+}
+
+// ------------------------------------------------------------------------
+
+// Producer number of a warp that is neither epilogue nor MMA (4, 8): first the
+// warps of the three schedulers without MMA warps (warp mod 4 = 1, 2, 3).
+__device__ __forceinline__ int prod_index(int warp)
+{
+    return (warp & 3) ? 3 * ((warp >> 2) - 1) + (warp & 3) - 1 : 9;
+}
+
+template <int N2>
+__global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const __grid_constant__ BatchLaunch b)
+{
+    using L = Tens<N2>;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);  // [kStages] stage written
+    uint64_t* empty = full + kStages;                                 // [kStages] stage read by the MMAs
+    uint64_t* accfull = empty + kStages;                                // [2] accumulator finished
+    uint64_t* accempty = accfull + 2;                                 // [2] accumulator read
+    uint64_t* drain = accempty + 2;
+    uint64_t* psync = drain + 2;                                      // the producer warps among themselves
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(psync + 1);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&accfull[i], 1);
+            mbar_init(&accempty[i], 4);
+        }
+        mbar_init(&drain[0], 1);
+        mbar_init(&drain[1], 1);
+        mbar_init(psync, kProd);
+        *s_abort = 0;
+        mbar_fence_init();
+    }
+    if (warp == 4) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "n"(L::ALLOC)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    bool timed_out = false;
+
+    if (warp < 4) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
+    else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
+    if (warp < 4) {
+        // ---------------- epilogue ----------------
+        const int row = warp * 32 + lane;
+        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+        long long fb = 0;
+        bool stop = false;
+        for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
+            if (*s_abort) break;
+            const TItem it = tensor_item(b, item);
+            if (!it.ok) continue;
+            const int ft = min(kFoldTiles, it.f->flush_tiles);
+            float2 s[L::N / 2], e[L::N / 2];
+#pragma unroll
+            for (int c = 0; c < L::N / 2; ++c) s[c] = e[c] = make_float2(0.f, 0.f);
+            const float2 neg = make_float2(-1.f, -1.f);
+            for (int t = 0; t < it.nt; t += ft, ++fb) {
+                const int buf = (int)(fb & 1);
+                if (field_wait(&accfull[buf], (unsigned)((fb >> 1) & 1), s_abort, b.abort, timed_out) != WAIT_DONE) {
+                    stop = true;
+                    break;
+                }
+                tc_fence_after();
+                const float ub = 1.f + 1.1920929e-7f * (float)(min(ft, it.nt - t) - 1);  // see Precision above
+                const float2 unb = make_float2(ub, ub);
+                const uint32_t base = lane_base + buf * L::DCOLS;
+#pragma unroll
+                for (int blk = 0; blk < L::NP / 8; ++blk) {
+                    uint32_t h[8], x[8];
+                    tmem_ld8(base + blk * 8, h);
+                    tmem_ld8(base + L::NP + blk * 8, x);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int c = blk * 4 + i;
+                        if (c < L::N / 2) {
+                            const float2 v = __ffma2_rn(
+                                make_float2(__uint_as_float(h[2 * i]), __uint_as_float(h[2 * i + 1])), unb,
+                                make_float2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])));
+                            // Kahan: the running sum is s - e
+                            const float2 y = __ffma2_rn(e[c], neg, v);
+                            const float2 u = __fadd2_rn(s[c], y);
+                            e[c] = __ffma2_rn(y, neg, __ffma2_rn(s[c], neg, u));
+                            s[c] = u;
+                        }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&accempty[buf]);
+            }
+            if (!stop) write_item<N2>(it, row, s, e);
+        }
+    } else if (warp == 4 || warp == 8) {
+        // ---------------- MMA issue ----------------
+        // The whole warp runs the loop and every condition and loaded value is
+        // made warp-uniform by a vote or a broadcast, so that descriptors and
+        // addresses live in uniform registers, where the MMA takes them from;
+        // one elected lane issues.  Issued from a one-lane branch each MMA cost
+        // about 200 cycles.  Two warps, one per accumulator: a tile's barrier,
+        // four MMAs and commit take one warp over 400 cycles, most of them
+        // latency, and the producers make a tile in 440.
+        const unsigned mine = warp == 8;
+        constexpr unsigned kAll = 0xffffffffu;
+        const uint64_t ah0 = smem_desc(smem_u32(smem));
+        unsigned fb = 0;  // run number: accumulator fb & 1, its stages' phase fb >> 1
+        bool go = true;
+        for (long long item = blockIdx.x; item < b.n_items && go; item += gridDim.x) {
+            if (__any_sync(kAll, launch_aborted(b, s_abort))) break;
+            const TItem it = tensor_item(b, item);
+            const int nt = __shfl_sync(kAll, it.ok ? it.nt : 0, 0);
+            const int ft = __shfl_sync(kAll, min(kFoldTiles, it.f->flush_tiles), 0);
+            for (int t = 0; t < nt && go; t += ft, ++fb) {
+                const unsigned buf = fb & 1, use = (fb >> 1) & 1;
+                if (buf != mine) continue;
+                // the accumulator's last run has been read (the first two waits pass at once)
+                go = __all_sync(kAll, field_wait(&accempty[buf], use ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE);
+                if (!go) break;
+                const uint32_t d = tmem + buf * L::DCOLS;
+                const uint64_t ab = ah0 + buf * (kFoldTiles * (L::STAGE >> 4));
+                uint64_t* fullb = full + buf * kFoldTiles;
+                uint64_t* emptyb = empty + buf * kFoldTiles;
+                const int cnt = min(ft, nt - t);
+                bool ready = mbar_test(&fullb[0], use);
+#pragma unroll
+                for (int i = 0; i < kFoldTiles; ++i) {
+                    if (!__all_sync(kAll, ready))
+                        go = __all_sync(kAll,
+                                        field_wait(&fullb[i], use, s_abort, b.abort, timed_out) == WAIT_DONE);
+                    if (!go) break;
+                    if (i + 1 < kFoldTiles) ready = mbar_test(&fullb[i + 1], use);  // asked for ahead
+                    tc_fence_after();
+                    const uint64_t ah = ab + i * (L::STAGE >> 4);
+                    const uint64_t al = ah + (kABytes >> 4), bh = ah + (2 * kABytes >> 4);
+                    if (elect_one()) {
+                        if (i < cnt) {
+                            mma_f16(d, ah, bh, mma_idesc(2 * L::NP), i > 0);            // hi (hi | lo)
+                            mma_f16(d + L::NP, al, bh, mma_idesc(L::NC), 1);            // lo hi
+                            mma_f16(d, ah + 16, bh + 16, mma_idesc(2 * L::NP), 1);      // nodes 16..31
+                            mma_f16(d + L::NP, al + 16, bh + 16, mma_idesc(L::NC), 1);
+                        }
+                        mma_commit(&emptyb[i]);
+                        if (i + 1 == kFoldTiles) mma_commit(&accfull[buf]);
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        // no MMA may be in flight when the tensor memory is freed
+        if (elect_one()) mma_commit(&drain[mine]);
+        __syncwarp();
+        if (mbar_wait(&drain[mine], 0) != WAIT_DONE) timed_out = true;
+    } else if (prod_index(warp) < kProd) {
+        // ---------------- producers ----------------
+        const int w = prod_index(warp);  // and its stage
+        const unsigned half = w / kFoldTiles;
+        const int slot = w % kFoldTiles;
+        unsigned fb0 = 0;     // runs of this CTA's items so far
+        bool stop = false;
+        ProdSync ps{psync, s_abort, b.abort, 0, false};
+        for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
+            if (*s_abort) break;
+            const TItem it = tensor_item(b, item);
+            if (!it.ok) {
+                // the MMAs may still read the stage this warp borrows: its last run
+                // was the newest one on its half
+                const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
+                if (fb0 > half && field_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out) != WAIT_DONE)
+                    break;
+                if (!plain_item<N2>(smem, it, w, lane, ps)) break;
+                continue;
+            }
+            const int nseg = segments(it.f->n_omega, N2);
+            const TensorSteps steps = it.f->steps;
+            // this warp's stage is number `slot` of every second run; a short run
+            // leaves it without a tile, and it is then only passed on
+            const int ft = min(kFoldTiles, it.f->flush_tiles);
+            const int nruns = (it.nt + ft - 1) / ft;
+            auto tile_of = [&](int r) {
+                const int t = r * ft + slot;
+                return r < nruns && slot < ft && t < it.nt ? t : -1;
+            };
+            float nd[9];
+            int r = (int)((fb0 ^ half) & 1), t = tile_of(r);
+            if (t >= 0) load_node(*it.f, it.t0 + t, lane, nd);
+            for (; r < nruns; r += 2) {
+                float cur[9];
+#pragma unroll
+                for (int f = 0; f < 9; ++f) cur[f] = nd[f];
+                const int tr = t;
+                t = tile_of(r + 2);
+                if (t >= 0) load_node(*it.f, it.t0 + t, lane, nd);
+                // the MMAs have read the stage's last contents (the first use passes at once)
+                const unsigned use = ((fb0 + r) >> 1) & 1;
+                auto stage_free = [&] {
+                    return field_wait(&empty[w], use ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE;
+                };
+                if (!(tr >= 0 ? produce_tile<N2>(smem + w * L::STAGE, cur, it, lane, nseg, steps, stage_free)
+                              : stage_free())) {
+                    stop = true;
+                    break;
+                }
+                fence_proxy_async();  // this lane's operand stores, before the MMAs read them
+                __syncwarp();
+                if (lane == 0 && !skip_copy(b, item, tr)) mbar_arrive(&full[w]);
+            }
+            fb0 += nruns;
+        }
+        timed_out |= ps.timed_out;
+    }
+    if (timed_out) atomicOr(b.err, ERR_TIMEOUT);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 4) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(L::ALLOC));
+    }
+}
+
+float2 ff(double w)
+{
+    const float hi = (float)w;
+    return make_float2(hi, (float)(w - (double)hi));
+}
+
+template <int N2>
+int launch_tensor(const BatchLaunch& b, int grid, cudaStream_t s)
+{
+    using L = Tens<N2>;
+    auto kern = field_tensor_kernel<N2>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM);
+    if (e != cudaSuccess) return -(int)e;
+    kern<<<grid, kTensorThreads, L::SMEM, s>>>(b);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? 1 : -(int)e;
+}
+
+}  // namespace
+
+int tensor_class(int n_omega)
+{
+    if (n_omega < kTensorMinOmega || n_omega > kTensorMaxOmega) return -1;
+    return n_omega <= 2 * kRows ? kFirstTensorClass : kFirstTensorClass + 1;
+}
+
+void tensor_prepare(int cls, FieldLaunch& f)
+{
+    const int n2 = cls == kFirstTensorClass ? 2 : 4;
+    const double om0 = (double)f.om_hi0 + (double)f.om_lo0, dom = (double)f.dom_hi + (double)f.dom_lo;
+    const double seed_row = 8 * seed_seg(segments(f.n_omega, n2)) + 3;
+    f.steps.seed = ff(om0 + (seed_row * n2 + 0.5 * (n2 - 1)) * dom);
+    f.steps.row = ff(n2 * dom);
+    f.steps.seg = ff(8 * n2 * dom);
+    f.steps.col = ff((n2 & 1) ? dom : 0.5 * dom);
+    f.steps.k0 = ff(6.283185307179586 * om0);
+    f.steps.dk = ff(6.283185307179586 * dom);
+}
+
+void tensor_field_shape(int cls, int device, int* ppc, int* slots)
+{
+    *ppc = 1;
+    *slots = cls == kFirstTensorClass
+                 ? resident(field_tensor_kernel<2>, kTensorThreads, Tens<2>::SMEM, device)
+                 : resident(field_tensor_kernel<4>, kTensorThreads, Tens<4>::SMEM, device);
+}
+
+int launch_tensor_field(int cls, const BatchLaunch& b, int grid, cudaStream_t s)
+{
+    return cls == kFirstTensorClass ? launch_tensor<2>(b, grid, s) : launch_tensor<4>(b, grid, s);
+}
+
+}  // namespace sc

@@ -77,6 +77,7 @@ struct TablePart {
     int n_rim_tiles = 0;
     const sc::Node64* d64 = nullptr;  // surface records, then rim records
     int n_rim = 0;
+    float amax_surf = 0.f, amax_rim = 0.f;  // largest |J|, |rho| of its surface and rim nodes
 };
 
 struct Table {
@@ -86,6 +87,7 @@ struct Table {
     sc::Node64* d64 = nullptr;     // and one for their FP64 records
     int n_surf = 0, n_rim = 0;
     std::vector<TablePart> parts;
+    float pmin = 0.f;              // smallest |P| of the surface and rim nodes
     double kc = 0.0, kh = 1.0;     // Chebyshev band in k of the CHEB parts
     bool fp32_ok = true;           // the incident wavefront focuses on the origin, so the
                                    // compensated FP32 phase is exact (else FP64 only)

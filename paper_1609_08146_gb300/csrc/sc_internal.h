@@ -36,6 +36,15 @@ enum : int { ERR_TIMEOUT = 1, ERR_NEAR_SURFACE = 2, ERR_NONFINITE = 4 };
 // B (re, im) x 3.
 constexpr int kAcc = 12;
 
+// Phases of the tensor kernel's operands as float-float pairs, in omegas: the
+// centre of the seed row phasor, the steps from row to row and from one segment
+// of eight rows to the next, the smallest column offset; and k of the first
+// omega and its step (tensor_prepare fills them).
+struct TensorSteps {
+    float2 seed, row, seg, col;
+    float2 k0, dk;
+};
+
 struct FieldLaunch {
     const float* nodes;     // tiled table: surface tiles then rim tiles
     int n_surf_tiles;
@@ -50,6 +59,10 @@ struct FieldLaunch {
     float dom_hi, dom_lo;   // grid step as a float-float pair
     float2* ws;             // compensated partials (hi, lo) [n_splits + 1][n_pts][n_omega][kAcc]
     int* err;               // device error word
+    // bounds for the tensor kernel's operand scaling (sc_field_tensor.cu): the
+    // largest |J|, |rho| of the table's surface and rim nodes, the smallest |P|
+    float amax_surf = 0.f, amax_rim = 0.f, pmin = 0.f;
+    TensorSteps steps{};
 };
 
 // One request (or one chunk of a request) of a batched field-sum launch:
@@ -87,10 +100,12 @@ struct BatchLaunch {
 // Kernel class for a chunk of n_omega (<= 2048) omegas: 0..20 the direct
 // kernel (1 to 32 threads per point, 1..8 omegas per thread, up to 256
 // omegas), 21..23 the grouped kernel with 64, 128, 256 threads per point,
-// 24..29 alternative direct layouts for the autotuner.
-constexpr int kNumClasses = 30;
+// 24..29 alternative direct layouts for the autotuner, 30, 31 the tensor
+// kernel with 2 and 4 omegas per row phasor (up to 128 and 256 omegas).
+constexpr int kNumClasses = 32;
 constexpr int kFirstGroupedClass = 21;  // grouped classes 21..23
 constexpr int kFirstAltClass = 24;      // alternative direct layouts 24..29 (alt_field_class)
+constexpr int kFirstTensorClass = 30;
 int field_class(int n_omega);
 // The alternative direct layout the autotuner times against field_class(n)
 // for n omegas, or -1 where there is none: 8 omegas on one thread of 8
@@ -99,7 +114,18 @@ int field_class(int n_omega);
 int alt_field_class(int n_omega);
 // Threads per point and omegas per thread of a class.
 void class_layout(int cls, int* threads_per_point, int* omegas_per_thread);
-inline bool is_direct_class(int cls) { return cls < kFirstGroupedClass || cls >= kFirstAltClass; }
+inline bool is_tensor_class(int cls) { return cls >= kFirstTensorClass; }
+inline bool is_direct_class(int cls)
+{
+    return cls < kFirstGroupedClass || (cls >= kFirstAltClass && !is_tensor_class(cls));
+}
+// Tensor class of a chunk, or -1 where the FP32 kernels keep it
+// (sc_field_tensor.cu); its shape and launch.
+constexpr int kTensorMinOmega = 25, kTensorMaxOmega = 256;
+int tensor_class(int n_omega);
+void tensor_prepare(int cls, FieldLaunch& f);  // fills f.steps
+void tensor_field_shape(int cls, int device, int* points_per_item, int* resident_ctas);
+int launch_tensor_field(int cls, const BatchLaunch& b, int grid, cudaStream_t s);
 // the direct kernel's classes (0 .. kFirstGroupedClass - 1), in sc_field_direct.cu
 void direct_field_shape(int cls, int device, int* points_per_item, int* resident_ctas);
 int launch_direct_field(int cls, const BatchLaunch& b, int grid, cudaStream_t s);

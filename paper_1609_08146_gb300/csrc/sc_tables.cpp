@@ -851,6 +851,19 @@ sc_status get_table(sc_ctx* ctx, const sc_mirror_t* m, const sc_incident_t* in, 
         tp.n_rim_tiles = rim_tiles[i];
         tp.d64 = t.d64 + off64[i];
         tp.n_rim = (int)hp[i].rim.size();
+        double pmin = i == 0 ? 1e300 : (double)t.pmin;
+        auto bound = [&](const std::vector<HostNode>& v) {
+            double a = 0.0;
+            for (const auto& nd : v) {
+                a = std::max(a, std::max(sqrt(nd.jx * nd.jx + nd.jy * nd.jy + nd.jz * nd.jz), fabs(nd.rho)));
+                if (!std::isfinite(nd.jx + nd.jy + nd.jz + nd.rho)) a = 1e300;
+                pmin = std::min(pmin, nd.pn);
+            }
+            return (float)std::min(a, 1e38);
+        };
+        tp.amax_surf = bound(hp[i].surf);
+        tp.amax_rim = bound(hp[i].rim);
+        t.pmin = (float)std::min(pmin, 1e38);
         t.parts.push_back(tp);
     }
     e = cudaMemcpyAsync(t.d32, t32.data(), b32, cudaMemcpyHostToDevice, stream);
