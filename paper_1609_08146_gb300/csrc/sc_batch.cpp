@@ -41,10 +41,13 @@ int heuristic_splits(int tiles, long long pb, int slots, double item_evals)
 {
     // enough items for dynamic balance (about 16 per resident CTA), items of
     // at most kMaxItemEvals evaluations and at least 32 node tiles, at most
-    // 64 splits
+    // 64 splits; where that leaves CTAs without an item, smaller items (two
+    // tiles at least) until each has one: 1024 points x 64^2 nodes x 1 omega
+    // ran on 20 CTAs, now on 260
     long long s = (16LL * slots + pb - 1) / pb;
     s = std::max<long long>(s, (long long)std::ceil(item_evals / kMaxItemEvals));
-    s = std::min<long long>(s, std::max(1, tiles / 32));
+    const long long wave = std::min<long long>(std::max(1, tiles / 2), (slots + pb - 1) / pb);
+    s = std::min<long long>(s, std::max<long long>(std::max(1, tiles / 32), wave));
     return (int)std::max<long long>(1, std::min<long long>(64, s));
 }
 
@@ -400,7 +403,7 @@ sc_status launch_chunks(sc_ctx* ctx, Lane& ln, std::vector<Chunk>& ch, float2* w
         c.rl.ws = ws + off;
         c.rl.off = roff;
         off += c.ws_elems;
-        roff += (long long)c.rl.n_pts * c.rl.n_omega;
+        roff += sc::reduce_size(c.rl);
     }
     if (off > ws_n) return fail(ctx, SC_ERR_OOM, "workspace plan exceeds its buffer");
     // per-class descriptor arrays

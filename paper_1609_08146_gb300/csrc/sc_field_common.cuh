@@ -335,14 +335,8 @@ __device__ __forceinline__ Item decode(const BatchLaunch& b, long long item)
     Item it;
     it.r = find_req(b, item);
     const long long local = item - it.r->item0;
-    if (local >> 32) {
-        it.pbi = (int)(local % it.r->pb);
-        it.split = (int)(local / it.r->pb);
-    } else {  // a 64-bit division costs over a hundred instructions
-        const unsigned l = (unsigned)local, pb = (unsigned)it.r->pb;
-        it.split = (int)(l / pb);
-        it.pbi = (int)(l - (unsigned)it.split * pb);
-    }
+    it.pbi = (int)(local % it.r->pb);
+    it.split = (int)(local / it.r->pb);
     return it;
 }
 

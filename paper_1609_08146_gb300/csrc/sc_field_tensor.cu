@@ -207,7 +207,17 @@ struct TItem {
 
 __device__ __forceinline__ TItem tensor_item(const BatchLaunch& b, long long item)
 {
-    const Item w = decode(b, item);
+    // decode(), with a 32-bit division where it can be (every role of every
+    // item pays for it; the 64-bit one takes over a hundred instructions)
+    Item w;
+    w.r = find_req(b, item);
+    const long long local = item - w.r->item0;
+    if (local >> 32) {
+        w = decode(b, item);
+    } else {
+        w.split = (int)((unsigned)local / (unsigned)w.r->pb);
+        w.pbi = (int)((unsigned)local % (unsigned)w.r->pb);
+    }
     TItem t;
     t.f = &w.r->f;
     t.pt = w.pbi;

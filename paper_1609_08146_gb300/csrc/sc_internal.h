@@ -154,11 +154,12 @@ struct ReduceLaunch {
     float2* E;              // output base (already offset to the chunk)
     float2* B;              // nullable
     long long out_pt_stride_omega;  // n_pts_total * 3
-    long long off;          // prefix of n_pts * n_omega over a batch
+    long long off;          // prefix of reduce_size over a batch
 };
 int launch_reduce_f32(const ReduceLaunch& p, cudaStream_t s);
+long long reduce_size(const ReduceLaunch& p);  // its threads
 // Reduction of many requests in one launch: reqs is a device array sorted
-// by off, total = sum of n_pts * n_omega.
+// by off, total = sum of their reduce_size.
 int launch_reduce_batch(const ReduceLaunch* reqs, int n_req, long long total, cudaStream_t s);
 
 // Plain FP64 path: direct sincos per (point, node, omega).
