@@ -315,6 +315,21 @@ static void fill_shape(sc_eval_stats* st, int cls, int splits)
     }
 }
 
+// The step of a wavenumber grid that is uniform to rounding over any eight
+// neighbours (k_{n+j} = k_n + j dk to about an ulp or two, j < 8), else 0: the
+// FP64 kernel then rotates a thread's first phasor through its omegas.
+static double rotation_step(const std::vector<double>& k)
+{
+    const int n = (int)k.size();
+    if (n < 2) return 0.0;
+    const double dk = (k[n - 1] - k[0]) / (n - 1);
+    if (!(dk > 0.0)) return 0.0;
+    for (int i = 0; i < n; ++i)
+        for (int j = 1; j < 8 && i + j < n; ++j)
+            if (fabs(k[i + j] - (k[i] + j * dk)) > 4.5e-16 * k[n - 1]) return 0.0;
+    return dk;
+}
+
 static sc_status eval_unlocked(sc_ctx* ctx, const sc_mirror_t* m, const sc_incident_t* in,
                                const double* omegas, int n_omega, const double* points_xyz,
                                int n_points, sc_precision prec, double dom, void* E_out,
@@ -391,17 +406,25 @@ static sc_status eval_unlocked(sc_ctx* ctx, const sc_mirror_t* m, const sc_incid
             f1 = take_event(ctx);
             cudaEventRecord(f0, ctx->stream);
         }
+        sc::Field64Launch a;
+        a.n_surf = tab->n_surf;
+        a.pts = d_pts;
+        a.n_pts = n_points;
+        a.kval = d_k;
+        a.n_omega = n_omega;
+        a.dk = rotation_step(kv);
+        sc::plan_field_f64(a, ctx->device);
+        if (const size_t need = sc::field_f64_workspace(a)) {
+            // a workspace over the budget costs speed, not the call
+            if (ctx->budget && ctx->main.ws.n < need && ctx->held - ctx->main.ws.n + need > ctx->budget) a.n_splits = 1;
+            else if ((st = ensure(ctx, ctx->main.ws, need)) != SC_OK) return st;
+            a.ws = (double*)ctx->main.ws.p;
+        }
         for (size_t p = 0; p < tab->parts.size(); ++p) {
             const TablePart& tp = tab->parts[p];
-            sc::Field64Launch a;
             a.surf = tp.d64;
-            a.n_surf = tab->n_surf;
             a.rim = tp.d64 + tab->n_surf;
             a.n_rim = tp.n_rim;
-            a.pts = d_pts;
-            a.n_pts = n_points;
-            a.kval = d_k;
-            a.n_omega = n_omega;
             a.amp = d_amp + p * 2 * (size_t)n_omega;
             a.E = (double2*)dE;
             a.B = (double2*)dB;

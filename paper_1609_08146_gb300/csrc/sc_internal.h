@@ -171,7 +171,14 @@ struct Field64Launch {
     const double* kval; int n_omega;     // k_n per omega
     const double* amp;                   // [n_omega][2]: a_n times the part's weight
     double2* E; double2* B;              // [n_omega][n_pts][3]
+    double dk = 0.0;                     // step of k where the grid is uniform to rounding, else 0
+    // plan (plan_field_f64): threads per point, omegas per thread, node splits;
+    // with several splits, ws holds [n_splits + 1][n_omega][n_pts][kAcc] sums
+    int gp = 1, nb = 1, n_splits = 1;
+    double* ws = nullptr;
 };
+void plan_field_f64(Field64Launch& p, int device);
+size_t field_f64_workspace(const Field64Launch& p);  // bytes of ws
 int launch_field_f64(const Field64Launch& p, cudaStream_t s);
 
 // Inverse transform: out[t][v] = 2 dk Re sum_n F[n][v] e^{-i k_n t_m}.
