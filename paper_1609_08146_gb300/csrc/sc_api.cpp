@@ -841,7 +841,9 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     for (int i = 0; i < n_omega; ++i) kv[i] = 2.0 * kPi * omegas[i];
     if ((st = ensure(ctx, ctx->tkval, kv.size() * sizeof(double))) != SC_OK) return st;
     if ((st = ensure(ctx, ctx->tvals, (size_t)n_t * sizeof(double))) != SC_OK) return st;
-    if ((st = ensure(ctx, ctx->phasor, (size_t)n_omega * n_t * sizeof(float2))) != SC_OK) return st;
+    const bool tensor = sc::idft_on_tensor(n_omega, n_t);
+    if ((st = ensure(ctx, ctx->phasor, tensor ? sc::idft_scratch_bytes(n_omega, n_vals, n_t)
+                                              : (size_t)n_omega * n_t * sizeof(float2))) != SC_OK) return st;
     const void* dEs = E_spec;
     const void* dBs = B_spec;
     if (!in_dev) {
@@ -863,20 +865,27 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     }
     SC_CUDA(cudaMemcpyAsync(ctx->tkval.p, kv.data(), kv.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->stream), "upload wavenumbers");
     SC_CUDA(cudaMemcpyAsync(ctx->tvals.p, times, (size_t)n_t * sizeof(double), cudaMemcpyHostToDevice, ctx->stream), "upload times");
-    for (int pass = 0; pass < (B_spec ? 2 : 1); ++pass) {
-        sc::IdftLaunch l;
+    sc::IdftLaunch l;
+    l.f64 = prec == SC_FP64;
+    l.n_omega = n_omega;
+    l.n_vals = n_vals;
+    l.kval = (const double*)ctx->tkval.p;
+    l.t = (const double*)ctx->tvals.p;
+    l.n_t = n_t;
+    l.dk = dk;
+    l.phasor = (float2*)ctx->phasor.p;
+    l.table = (unsigned char*)ctx->phasor.p;
+    l.dk_rot = rotation_step(kv);
+    l.err = ctx->d_err;
+    l.accumulate = accumulate;
+    for (int pass = 0; pass < (B_spec && !tensor ? 2 : 1); ++pass) {
         l.F = pass == 0 ? dEs : dBs;
-        l.f64 = prec == SC_FP64;
-        l.n_omega = n_omega;
-        l.n_vals = n_vals;
-        l.kval = (const double*)ctx->tkval.p;
-        l.t = (const double*)ctx->tvals.p;
-        l.n_t = n_t;
-        l.dk = dk;
         l.out = pass == 0 ? dEt : dBt;
-        l.phasor = (float2*)ctx->phasor.p;
-        l.accumulate = accumulate;
-        const int r = sc::launch_idft(l, ctx->stream);
+        if (tensor) {
+            l.F2 = dBs;
+            l.out2 = dBt;
+        }
+        const int r = tensor ? sc::launch_idft_tensor(l, ctx->stream) : sc::launch_idft(l, ctx->stream);
         if (r < 0) return cuda_fail(ctx, (cudaError_t)(-r), "inverse transform launch");
         ctx->ctr.launches += r;
     }

@@ -1,4 +1,5 @@
-// sc_f64_idft.cu -- the plain FP64 field sum and the inverse-transform stage.
+// sc_f64_idft.cu -- the plain FP64 field sum and the inverse transform of small
+// sizes (sc_idft.cu has the tensor-core kernel of the others).
 //
 // field_f64_kernel: the same quadrature of Sec. II Eq. 11 as the FP32 kernel,
 // written the plain way: FP64 throughout, phase R - (z + 2f) + W formed by a

@@ -58,7 +58,6 @@
 //               conflict-free); no data passes between lanes.
 // Items are strided over the CTAs (item = blockIdx + i gridDim), which every
 // role follows on its own; all waits are bounded as in the other kernels.
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -66,6 +65,7 @@
 
 #include "sc_field_common.cuh"
 #include "sc_internal.h"
+#include "sc_tensor.cuh"
 
 namespace sc {
 
@@ -99,95 +99,11 @@ struct Tens {
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-// ------------------------------------------------------------------------
-// tcgen05 wrappers
+// Stage layout, MN-major: 128 bytes from one block of 8 nodes to the next,
+// kBlkBytes from one block of 8 rows or columns to the next.
+__device__ __forceinline__ uint64_t stage_desc(uint32_t addr) { return smem_desc(addr, 128, kBlkBytes); }
 
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
-{
-    // no swizzle, MN-major: core matrices of 8 MN x 8 K; 128 bytes from one
-    // block of 8 K to the next (leading offset), kBlkBytes from one block of 8
-    // MN to the next (stride offset)
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(kBlkBytes >> 4) << 32) |
-           (1ull << 46);
-}
-
-// f16 x f16 -> f32, A and B MN-major, M = 128
-__host__ __device__ constexpr uint32_t mma_idesc(int n)
-{
-    return (1u << 4) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(2 * kRows >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t v[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(addr)
-                 : "memory");
-}
-
-// One look at an mbarrier's phase, without waiting.
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity)
-{
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
-    return p != 0;
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// ------------------------------------------------------------------------
-// Operand splitting: eight FP32 values -> eight fp16 (16 bytes) of the high
-// parts and eight of the low parts.
-
-__device__ __forceinline__ uint32_t pack_h2(float a, float b)
-{
-    const __half2 h = __floats2half2_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&h);
-}
-
-__device__ __forceinline__ void split_store8(unsigned char* hi, unsigned char* lo, const float2 x[4])
-{
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        h[i] = pack_h2(x[i].x, x[i].y);
-        float rx, ry;  // x - hi, exact (one mixed-precision FMA each)
-        asm("{\n\t.reg .b16 a, b, m;\n\tmov.b32 {a, b}, %2;\n\tmov.b16 m, 0xBC00;\n\t"
-            "fma.rn.f32.f16 %0, a, m, %3;\n\tfma.rn.f32.f16 %1, b, m, %4;\n\t}"
-            : "=f"(rx), "=f"(ry)
-            : "r"(h[i]), "f"(x[i].x), "f"(x[i].y));
-        l[i] = pack_h2(rx, ry);
-    }
-    *reinterpret_cast<uint4*>(hi) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(lo) = make_uint4(l[0], l[1], l[2], l[3]);
-}
+__host__ __device__ constexpr uint32_t stage_idesc(int n) { return mma_idesc(2 * kRows, n, true, true); }
 
 // Segments of eight row phasors that n_omega omegas take, and the one the
 // seeds start from (then outwards both ways).
@@ -669,7 +585,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         // latency, and the producers make a tile in 440.
         const unsigned mine = warp == 8;
         constexpr unsigned kAll = 0xffffffffu;
-        const uint64_t ah0 = smem_desc(smem_u32(smem));
+        const uint64_t ah0 = stage_desc(smem_u32(smem));
         unsigned fb = 0;  // run number: accumulator fb & 1, its stages' phase fb >> 1
         bool go = true;
         for (long long item = blockIdx.x; item < b.n_items && go; item += gridDim.x) {
@@ -701,10 +617,10 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                     const uint64_t al = ah + (kABytes >> 4), bh = ah + (2 * kABytes >> 4);
                     if (elect_one()) {
                         if (i < cnt) {
-                            mma_f16(d, ah, bh, mma_idesc(2 * L::NP), i > 0);            // hi (hi | lo)
-                            mma_f16(d + L::NP, al, bh, mma_idesc(L::NC), 1);            // lo hi
-                            mma_f16(d, ah + 16, bh + 16, mma_idesc(2 * L::NP), 1);      // nodes 16..31
-                            mma_f16(d + L::NP, al + 16, bh + 16, mma_idesc(L::NC), 1);
+                            mma_f16(d, ah, bh, stage_idesc(2 * L::NP), i > 0);            // hi (hi | lo)
+                            mma_f16(d + L::NP, al, bh, stage_idesc(L::NC), 1);            // lo hi
+                            mma_f16(d, ah + 16, bh + 16, stage_idesc(2 * L::NP), 1);      // nodes 16..31
+                            mma_f16(d + L::NP, al + 16, bh + 16, stage_idesc(L::NC), 1);
                         }
                         mma_commit(&emptyb[i]);
                         if (i + 1 == kFoldTiles) mma_commit(&accfull[buf]);

@@ -192,10 +192,22 @@ struct IdftLaunch {
     int n_t;
     double dk;
     float* out;             // [n_t][n_vals]
-    float2* phasor;         // scratch [n_omega][n_t]
+    const void* F2 = nullptr;  // a second spectrum and its output (B), or null
+    float* out2 = nullptr;
+    float2* phasor;         // scratch [n_omega][n_t] (FP32 kernel)
+    unsigned char* table = nullptr;  // scratch, idft_scratch_bytes (tensor kernel)
+    float* col_scale = nullptr;      // in it
+    double dk_rot = 0.0;    // step of k where the grid is uniform to rounding, else 0
+    int* err = nullptr;     // device error word
     int accumulate = 0;     // add to out (a later chunk of omegas) instead of storing
+    float scale = 0.f;      // 2 dk, and blocks of times (launch_idft_tensor fills them)
+    int m_blocks = 0;
 };
 int launch_idft(const IdftLaunch& p, cudaStream_t s);
+// The same on the tensor cores (sc_idft.cu), where that is the faster.
+bool idft_on_tensor(int n_omega, int n_t);
+size_t idft_scratch_bytes(int n_omega, long long n_vals, int n_t);
+int launch_idft_tensor(const IdftLaunch& p, cudaStream_t s);
 
 // First correction beyond physical optics (sc_mfie.cu): the current dJ of the
 // MFIE's Liouville-Neumann series at every surface node, by a polar rule about
