@@ -139,6 +139,7 @@ sc_status sc_destroy(sc_ctx* ctx)
     free_lane(ctx->main);
     for (cudaEvent_t e : ctx->pool) cudaEventDestroy(e);
     if (ctx->d_err) cudaFree(ctx->d_err);
+    if (ctx->d_trig) cudaFree(ctx->d_trig);
     if (ctx->h_err) cudaFreeHost(ctx->h_err);
     delete ctx;
     return SC_OK;
@@ -315,18 +316,17 @@ static void fill_shape(sc_eval_stats* st, int cls, int splits)
     }
 }
 
-// The step of a wavenumber grid that is uniform to rounding over any eight
-// neighbours (k_{n+j} = k_n + j dk to about an ulp or two, j < 8), else 0: the
-// FP64 kernel then rotates a thread's first phasor through its omegas.
+// The step of a wavenumber grid that is uniform to rounding (k_n = k_0 + n dk to
+// two units in the last place of the largest), else 0: the FP64 kernel and the
+// phase table then rotate phase factors from one omega to the next.
 static double rotation_step(const std::vector<double>& k)
 {
     const int n = (int)k.size();
     if (n < 2) return 0.0;
     const double dk = (k[n - 1] - k[0]) / (n - 1);
     if (!(dk > 0.0)) return 0.0;
-    for (int i = 0; i < n; ++i)
-        for (int j = 1; j < 8 && i + j < n; ++j)
-            if (fabs(k[i + j] - (k[i] + j * dk)) > 4.5e-16 * k[n - 1]) return 0.0;
+    for (int i = 1; i < n; ++i)
+        if (fabs(k[i] - (k[0] + i * dk)) > 4.5e-16 * k[n - 1]) return 0.0;
     return dk;
 }
 
@@ -413,6 +413,18 @@ static sc_status eval_unlocked(sc_ctx* ctx, const sc_mirror_t* m, const sc_incid
         a.kval = d_k;
         a.n_omega = n_omega;
         a.dk = rotation_step(kv);
+        if (!ctx->d_trig) {
+            // made on first use (16 KB beside the budget, as the error word is)
+            double2* tab = nullptr;
+            SC_CUDA(cudaMalloc(&tab, sc::kTrigEntries * sizeof(double2)), "trigonometric table");
+            const int r = sc::launch_trig_table(tab, ctx->stream);
+            if (r < 0) {
+                cudaFree(tab);
+                return cuda_fail(ctx, (cudaError_t)(-r), "trigonometric table launch");
+            }
+            ctx->d_trig = tab;
+        }
+        a.trig = ctx->d_trig;
         sc::plan_field_f64(a, ctx->device);
         if (const size_t need = sc::field_f64_workspace(a)) {
             // a workspace over the budget costs speed, not the call

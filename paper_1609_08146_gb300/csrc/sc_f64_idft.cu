@@ -7,17 +7,19 @@
 // baseline.  An incident with several node tables runs once per table, the
 // later ones adding to E and B.
 //
-// What bounds it: FP64 instructions, 2 a cycle and SM.  A term needs 22 of them
-// (q, z and 18 sums); one thread per (point, omega) paid some 90 more for the
-// pair's geometry (a square root, a division) and a sincos.  Now gp threads of
-// NB omegas share a point: each computes the pair of one node of every gp into
-// shared memory, all of them read it, and a thread takes one sincos per pair,
-// for its first omega, and rotates it through the others (4 instructions, on
-// grids uniform to rounding; others keep a sincos per omega).  512 points x
-// 128^2 nodes x 64 omegas: 103.8 -> 37.1 ms.  Where points and omegas are too
-// few for the chip the nodes are split over the grid and the splits' sums added
-// by a second kernel: 1024 points x 64^2 nodes x 1 omega, 8 blocks before:
-// 13.65 -> 0.87 ms.
+// What bounds it: FP64 instructions, 2 a cycle and SM.  A term needs 21 of them
+// (a phase factor's two forms and 18 sums); one thread per (point, omega) paid
+// some 90 more for the pair's geometry (a square root, a division) and a sincos.
+// Now gp threads of NB omegas share a point: each computes the pair of one node
+// of every gp, and the first phase factor of every thread for it, into shared
+// memory; all of them read it and go on from their first two factors by the
+// three-term recurrence (on grids uniform to rounding; others take a sincos per
+// omega).  Sine and cosine come from a table and short polynomials (16
+// instructions).  512 points x 128^2 nodes x 64 omegas: 103.6 ms with a thread per
+// (point, omega), 37.1 with shared pairs, a sincos per thread and rotations, now
+// 30.2.  Where points and omegas are too few for the chip the nodes are split
+// over the grid and the splits' sums added by a second kernel: 1024 points x
+// 64^2 nodes x 1 omega, 8 blocks at first: 13.65 ms, 0.85 with splits, now 0.77.
 //
 // idft: Sec. III.B Eq. 13 for a real field sampled at positive k_n,
 // F(t_m) = 2 dk Re sum_n F_n e^{-i k_n t_m}, as a phasor table
@@ -35,7 +37,45 @@ namespace sc {
 namespace {
 
 constexpr int kF64Threads = 128;
-constexpr int kF64Row = 13;  // doubles per shared pair row: ir, phi, rotation, U, V, Wv
+constexpr int kF64Row = 13;  // doubles per shared pair row: ir, phi, U, V, Wv, rotation e^{i dk Phi}
+                             // (and then the threads' first phase factors)
+
+// sin and cos by table lookup (P. T. P. Tang, "Table-lookup algorithms for
+// elementary functions and their error analysis", 1991): x = j 2 pi / N + r with
+// |r| <= pi / N, the N pairs (cos, sin)(2 pi j / N) from memory and Taylor
+// polynomials of sin r and cos r - 1 (the first terms left out are below 2^-60 for
+// N = 1024).  16 FP64 instructions; sincos() takes about 37.  Arguments from 2^30
+// on, infinities and NaN go to sincos().
+constexpr int kTrigN = kTrigEntries;
+constexpr double kTrigStepLo = 2.391888279584674e-19;  // 2 pi / N beyond its double
+
+__device__ __forceinline__ void sincos_tab(const double2* tab, double x, double* sn, double* cs)
+{
+    if ((__double2hiint(x) & 0x7fffffff) >= 0x41d00000) {
+        sincos(x, sn, cs);
+        return;
+    }
+    constexpr double kMagic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the nearest integer
+    const double t = fma(x, 162.97466172610083, kMagic);  // N / (2 pi)
+    const double j = t - kMagic;
+    double r = fma(j, -0.006135923151542565, x);           // 2 pi / N, and what the double leaves of it
+    r = fma(j, -kTrigStepLo, r);
+    const double2 cS = __ldg(tab + (__double2loint(t) & (kTrigN - 1)));
+    const double r2 = r * r;
+    const double sr = fma(r * r2, fma(r2, 1.0 / 120.0, -1.0 / 6.0), r);
+    const double cm = r2 * fma(r2, 1.0 / 24.0, -0.5);
+    *sn = cS.y + fma(cS.y, cm, cS.x * sr);
+    *cs = cS.x + fma(cS.x, cm, -cS.y * sr);
+}
+
+__global__ void trig_table_kernel(double2* tab)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= kTrigN) return;
+    double s, c;
+    sincospi(2.0 * j / kTrigN, &s, &c);
+    tab[j] = make_double2(c, s);
+}
 
 // One pair's geometry: row = {1/R, Phi, U[3], V[3], Wv[3]}.
 __device__ __forceinline__ void pair64(const Node64& nd, double x, double y, double z, double row[11])
@@ -55,17 +95,29 @@ __device__ __forceinline__ void pair64(const Node64& nd, double x, double y, dou
     row[10] = ux * ry - uy * rx;
 }
 
-// E += U q + V z, B += Wv z with ph = (c, s), q = ik ph, z = q - ph/R.
-__device__ __forceinline__ void eval64(double sE[6], double sB[6], const double* row, double k, double c, double s)
+// Without the common factor ik: E' += U ph + V y, B' += Wv y with ph = (c, s) and
+// y = (1 + i / (kR)) ph; w = 1 / (kR).
+__device__ __forceinline__ void eval64(double sE[6], double sB[6], const double* row, double ik, double c, double s)
 {
-    const double qr = -k * s, qi = k * c;
-    const double zr = qr - row[0] * c, zi = qi - row[0] * s;
+    const double w = row[0] * ik;
+    const double yr = c - w * s, yi = s + w * c;
 #pragma unroll
     for (int cc = 0; cc < 3; ++cc) {
-        sE[2 * cc] += row[2 + cc] * qr + row[5 + cc] * zr;
-        sE[2 * cc + 1] += row[2 + cc] * qi + row[5 + cc] * zi;
-        sB[2 * cc] += row[8 + cc] * zr;
-        sB[2 * cc + 1] += row[8 + cc] * zi;
+        sE[2 * cc] += row[2 + cc] * c + row[5 + cc] * yr;
+        sE[2 * cc + 1] += row[2 + cc] * s + row[5 + cc] * yi;
+        sB[2 * cc] += row[8 + cc] * yr;
+        sB[2 * cc + 1] += row[8 + cc] * yi;
+    }
+}
+
+// ik times a node range's sums
+__device__ __forceinline__ void times_ik(double s[6], double k)
+{
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+        const double re = s[2 * cc];
+        s[2 * cc] = -k * s[2 * cc + 1];
+        s[2 * cc + 1] = k * re;
     }
 }
 
@@ -95,47 +147,102 @@ __device__ __forceinline__ void finish64(const Field64Launch& a, int n, int pt, 
 }
 
 // Sum the nodes [j0, j1) into NB omegas' E and B.  gp threads (neighbouring
-// lanes, a power of two) of a point share its pairs through rows.
+// lanes, a power of two) of a point share its pairs through rows, `stride` doubles
+// each: kF64Row of the pair and, with UNI, 2 gp of the threads' first phase factors.
 template <int NB, bool UNI>
 __device__ __forceinline__ void sum64(const Field64Launch& a, const Node64* nodes, int j0, int j1, double x, double y,
-                                      double z, int g, const double kv[NB], double (*rows)[kF64Row],
-                                      double (*sE)[6], double (*sB)[6])
+                                      double z, int g, double k0, const double kv[NB], const double ikv[NB],
+                                      double* rows, int stride, double (*sE)[6], double (*sB)[6])
 {
-    const int base = threadIdx.x - g;  // the point's first row
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) sE[i][c] = sB[i][c] = 0.0;
+    double* mine = rows + threadIdx.x * stride;
+    const double* base = rows + (threadIdx.x - g) * stride;  // the point's first row
     for (int j = j0; j < j1; j += a.gp) {
         double own[kF64Row];
+        double fs = 0.0, fc = 1.0;  // own first phase factor (gp = 1)
+        if (a.gp > 1) __syncwarp();  // the last round's rows are read
         if (j + g < j1) {
             pair64(nodes[j + g], x, y, z, own);
-            if (NB > 1 && UNI) sincos(a.dk * own[1], &own[12], &own[11]);
+            if (NB > 1 && UNI) sincos_tab(a.trig, a.dk * own[1], &own[12], &own[11]);
+            if (a.gp > 1) {
+#pragma unroll
+                for (int i = 0; i < kF64Row; ++i)
+                    if (i < 11 || (NB > 1 && UNI)) mine[i] = own[i];
+                if (UNI) {
+                    // e^{i (k0 + h NB dk) Phi} for every thread h of the point, by rotation
+                    // (k0: the first omega of the point's first thread)
+                    double rs, rc;
+                    sincos_tab(a.trig, k0 * own[1], &fs, &fc);
+                    sincos_tab(a.trig, NB * a.dk * own[1], &rs, &rc);
+                    for (int h = 0; h < a.gp; ++h) {
+                        reinterpret_cast<double2*>(mine + kF64Row + 1)[h] = make_double2(fc, fs);
+                        const double t = fc * rc - fs * rs;
+                        fs = fc * rs + fs * rc;
+                        fc = t;
+                    }
+                }
+            } else {
+                sincos_tab(a.trig, kv[0] * own[1], &fs, &fc);
+            }
         }
         const int m = min(a.gp, j1 - j);
-        if (a.gp > 1) {
-            __syncwarp();  // the last round's rows are read
-#pragma unroll
-            for (int i = 0; i < kF64Row; ++i) rows[threadIdx.x][i] = own[i];
-            __syncwarp();
-        }
+        if (a.gp > 1) __syncwarp();
         for (int q = 0; q < m; ++q) {
             double row[kF64Row];
+            if (a.gp > 1) {
+                const double* r = base + q * stride;
 #pragma unroll
-            for (int i = 0; i < kF64Row; ++i) row[i] = a.gp > 1 ? rows[base + q][i] : own[i];
-            double s, c;
-            sincos(kv[0] * row[1], &s, &c);
-            eval64(sE[0], sB[0], row, kv[0], c, s);
-#pragma unroll
-            for (int i = 1; i < NB; ++i) {
+                for (int i = 0; i < kF64Row; ++i)
+                    if (i < 11 || (NB > 1 && UNI)) row[i] = r[i];
                 if (UNI) {
-                    const double t = c * row[11] - s * row[12];
-                    s = c * row[12] + s * row[11];
-                    c = t;
+                    const double2 f = reinterpret_cast<const double2*>(r + kF64Row + 1)[g];
+                    fc = f.x;
+                    fs = f.y;
                 } else {
-                    sincos(kv[i] * row[1], &s, &c);
+                    sincos_tab(a.trig, kv[0] * row[1], &fs, &fc);
                 }
-                eval64(sE[i], sB[i], row, kv[i], c, s);
+            } else {
+#pragma unroll
+                for (int i = 0; i < kF64Row; ++i) row[i] = own[i];
+            }
+            eval64(sE[0], sB[0], row, ikv[0], fc, fs);
+            if (UNI && NB > 1) {
+                double c0 = fc, s0 = fs;
+                double c1 = fc * row[11] - fs * row[12], s1 = fc * row[12] + fs * row[11];
+                const double two = 2.0 * row[11];
+#pragma unroll
+                for (int i = 1; i < NB; ++i) {
+                    eval64(sE[i], sB[i], row, ikv[i], c1, s1);
+                    if (i + 1 < NB) {
+                        const double c2 = fma(two, c1, -c0), s2 = fma(two, s1, -s0);
+                        c0 = c1;
+                        s0 = s1;
+                        c1 = c2;
+                        s1 = s2;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int i = 1; i < NB; ++i) {
+                    double s, c;
+                    sincos_tab(a.trig, kv[i] * row[1], &s, &c);
+                    eval64(sE[i], sB[i], row, ikv[i], c, s);
+                }
             }
         }
     }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        times_ik(sE[i], kv[i]);
+        times_ik(sB[i], kv[i]);
+    }
 }
+
+// doubles of a shared row; a row's phase factors start on 16 bytes
+__host__ __device__ inline int f64_stride(int gp) { return gp > 1 ? kF64Row + 1 + 2 * gp : 0; }
 
 // blockIdx.x: points (128 / gp of them), y: omegas (gp NB of them), z: node
 // split.  One split sums surface and rim and writes the outputs; with several,
@@ -144,27 +251,28 @@ __device__ __forceinline__ void sum64(const Field64Launch& a, const Node64* node
 template <int NB, bool UNI>
 __global__ void __launch_bounds__(kF64Threads) field_f64_kernel(Field64Launch a)
 {
-    __shared__ double rows[kF64Threads][kF64Row];
+    extern __shared__ __align__(16) double rows[];
+    const int stride = f64_stride(a.gp);
     const int g = threadIdx.x % a.gp;
     const int pt = blockIdx.x * (kF64Threads / a.gp) + threadIdx.x / a.gp;
     const int n0 = (blockIdx.y * a.gp + g) * NB;
     const bool live = pt < a.n_pts;  // (idle lanes follow: their warp shares rows)
     const int p = live ? pt : a.n_pts - 1;
     const double x = a.pts[3 * p], y = a.pts[3 * p + 1], z = a.pts[3 * p + 2];
-    double kv[NB];
+    const double k0 = a.kval[min((int)blockIdx.y * a.gp * NB, a.n_omega - 1)];
+    double kv[NB], ikv[NB];
 #pragma unroll
-    for (int i = 0; i < NB; ++i) kv[i] = a.kval[min(n0 + i, a.n_omega - 1)];
+    for (int i = 0; i < NB; ++i) {
+        kv[i] = a.kval[min(n0 + i, a.n_omega - 1)];
+        ikv[i] = 1.0 / kv[i];
+    }
     double sE[NB][6], sB[NB][6];
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-#pragma unroll
-        for (int c = 0; c < 6; ++c) sE[i][c] = sB[i][c] = 0.0;
     if (a.n_splits > 1) {
         const bool rim = (int)blockIdx.z == a.n_splits;
         const int per = (a.n_surf + a.n_splits - 1) / a.n_splits;
         const int j0 = rim ? 0 : min((int)blockIdx.z * per, a.n_surf);
-        sum64<NB, UNI>(a, rim ? a.rim : a.surf, j0, rim ? a.n_rim : min(j0 + per, a.n_surf), x, y, z, g, kv, rows,
-                       sE, sB);
+        sum64<NB, UNI>(a, rim ? a.rim : a.surf, j0, rim ? a.n_rim : min(j0 + per, a.n_surf), x, y, z, g, k0, kv, ikv,
+                       rows, stride, sE, sB);
         if (!live) return;
 #pragma unroll
         for (int i = 0; i < NB; ++i)
@@ -180,16 +288,12 @@ __global__ void __launch_bounds__(kF64Threads) field_f64_kernel(Field64Launch a)
     }
     // one split: the rim's part of the outputs, then the surface's added to it
     const double zero[6] = {0, 0, 0, 0, 0, 0};
-    sum64<NB, UNI>(a, a.rim, 0, a.n_rim, x, y, z, g, kv, rows, sE, sB);
+    sum64<NB, UNI>(a, a.rim, 0, a.n_rim, x, y, z, g, k0, kv, ikv, rows, stride, sE, sB);
     if (live)
 #pragma unroll
         for (int i = 0; i < NB; ++i)
             if (n0 + i < a.n_omega) finish64(a, n0 + i, pt, zero, zero, sE[i], a.accumulate);
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-#pragma unroll
-        for (int c = 0; c < 6; ++c) sE[i][c] = sB[i][c] = 0.0;
-    sum64<NB, UNI>(a, a.surf, 0, a.n_surf, x, y, z, g, kv, rows, sE, sB);
+    sum64<NB, UNI>(a, a.surf, 0, a.n_surf, x, y, z, g, k0, kv, ikv, rows, stride, sE, sB);
     if (live)
 #pragma unroll
         for (int i = 0; i < NB; ++i)
@@ -326,9 +430,10 @@ void plan_field_f64(Field64Launch& a, int device)
     while (a.gp < 32 && a.n_omega > 6 * a.gp) a.gp *= 2;
     a.nb = a.n_omega >= 6 * a.gp ? 6 : (a.n_omega + a.gp - 1) / a.gp;
     int per_sm = 1, sms = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f64_kernel(a.nb, a.dk > 0.0), kF64Threads, 0) !=
-        cudaSuccess)
-        per_sm = 1;
+    const size_t smem = (size_t)kF64Threads * f64_stride(a.gp) * sizeof(double);
+    const F64Kernel kern = f64_kernel(a.nb, a.dk > 0.0);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kF64Threads, smem) != cudaSuccess) per_sm = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) sms = 1;
     cudaGetLastError();
     const int slots = std::max(1, per_sm) * std::max(1, sms);
@@ -341,6 +446,13 @@ void plan_field_f64(Field64Launch& a, int device)
     a.n_splits = (int)std::min<long long>(s, 1024);
 }
 
+int launch_trig_table(double2* tab, cudaStream_t s)
+{
+    trig_table_kernel<<<kTrigN / 128, 128, 0, s>>>(tab);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? 1 : -(int)e;
+}
+
 size_t field_f64_workspace(const Field64Launch& a)
 {
     return a.n_splits > 1 ? (size_t)(a.n_splits + 1) * a.n_omega * a.n_pts * kAcc * sizeof(double) : 0;
@@ -351,7 +463,8 @@ int launch_field_f64(const Field64Launch& a, cudaStream_t s)
     const int ppb = kF64Threads / a.gp, opb = a.gp * a.nb;
     const dim3 grid((unsigned)((a.n_pts + ppb - 1) / ppb), (unsigned)((a.n_omega + opb - 1) / opb),
                     (unsigned)(a.n_splits > 1 ? a.n_splits + 1 : 1));
-    f64_kernel(a.nb, a.dk > 0.0)<<<grid, kF64Threads, 0, s>>>(a);
+    const size_t smem = (size_t)kF64Threads * f64_stride(a.gp) * sizeof(double);
+    f64_kernel(a.nb, a.dk > 0.0)<<<grid, kF64Threads, smem, s>>>(a);  // (plan_field_f64 raised its limit)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return -(int)e;
     if (a.n_splits <= 1) return 1;

@@ -176,7 +176,10 @@ struct Field64Launch {
     // with several splits, ws holds [n_splits + 1][n_omega][n_pts][kAcc] sums
     int gp = 1, nb = 1, n_splits = 1;
     double* ws = nullptr;
+    const double2* trig = nullptr;       // kTrigEntries pairs (launch_trig_table)
 };
+constexpr int kTrigEntries = 1024;
+int launch_trig_table(double2* tab, cudaStream_t s);
 void plan_field_f64(Field64Launch& p, int device);
 size_t field_f64_workspace(const Field64Launch& p);  // bytes of ws
 int launch_field_f64(const Field64Launch& p, cudaStream_t s);
