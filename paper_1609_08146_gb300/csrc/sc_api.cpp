@@ -131,7 +131,7 @@ sc_status sc_destroy(sc_ctx* ctx)
     cudaStreamSynchronize(ctx->stream);
     settle_events(ctx);
     for (auto& t : ctx->tables) free_table(ctx, t);
-    for (DevBuf* b : {&ctx->pts, &ctx->outE, &ctx->outB, &ctx->tkval, &ctx->tvals, &ctx->phasor,
+    for (DevBuf* b : {&ctx->pts, &ctx->outE, &ctx->outB, &ctx->tkval, &ctx->phasor,
                       &ctx->specE, &ctx->specB, &ctx->tE, &ctx->tB, &ctx->fpts, &ctx->fspecE,
                       &ctx->fspecB, &ctx->ftE, &ctx->ftB, &ctx->mfie_geo, &ctx->mfie_zern, &ctx->mfie_gl,
                       &ctx->mfie_dJ})
@@ -372,12 +372,12 @@ static sc_status eval_unlocked(sc_ctx* ctx, const sc_mirror_t* m, const sc_incid
                                 cudaMemcpyHostToDevice, ctx->stream), "upload points");
         d_pts = (const double*)ctx->pts.p;
     }
+    // amplitudes, then wavenumbers, one upload
+    const size_t n_amp = amp.size();
+    amp.insert(amp.end(), kv.begin(), kv.end());
     if ((st = ensure(ctx, ctx->main.amp, amp.size() * sizeof(double))) != SC_OK) return st;
-    if ((st = ensure(ctx, ctx->main.kval, kv.size() * sizeof(double))) != SC_OK) return st;
     SC_CUDA(cudaMemcpyAsync(ctx->main.amp.p, amp.data(), amp.size() * sizeof(double),
-                            cudaMemcpyHostToDevice, ctx->stream), "upload amplitudes");
-    SC_CUDA(cudaMemcpyAsync(ctx->main.kval.p, kv.data(), kv.size() * sizeof(double),
-                            cudaMemcpyHostToDevice, ctx->stream), "upload wavenumbers");
+                            cudaMemcpyHostToDevice, ctx->stream), "upload amplitudes and wavenumbers");
 
     const size_t elem = prec == SC_FP64 ? sizeof(double2) : sizeof(float2);
     const size_t out_bytes = (size_t)n_omega * n_points * 3 * elem;
@@ -394,7 +394,7 @@ static sc_status eval_unlocked(sc_ctx* ctx, const sc_mirror_t* m, const sc_incid
     // the staging buffers may have moved: refresh pointers taken before
     if (!pts_dev) d_pts = (const double*)ctx->pts.p;
     const double* d_amp = (const double*)ctx->main.amp.p;
-    const double* d_k = (const double*)ctx->main.kval.p;
+    const double* d_k = d_amp + n_amp;
 
     const double evals = (double)n_points * (double)tab->n_surf * (double)n_omega;
     int shape_cls = -1, shape_splits = -1;  // reported in stats (FP32 path)
@@ -699,18 +699,17 @@ sc_status sc_eval_batch(sc_ctx* ctx, const sc_request* reqs, int n_req, sc_eval_
     }
     sc_status st;
     Lane& ln = ctx->main;
+    const size_t n_amp = amp_all.size();
+    amp_all.insert(amp_all.end(), k_all.begin(), k_all.end());
     if ((st = ensure(ctx, ln.amp, amp_all.size() * sizeof(double))) != SC_OK) return st;
-    if ((st = ensure(ctx, ln.kval, k_all.size() * sizeof(double))) != SC_OK) return st;
     SC_CUDA(cudaMemcpyAsync(ln.amp.p, amp_all.data(), amp_all.size() * sizeof(double),
-                            cudaMemcpyHostToDevice, ln.stream), "upload amplitudes");
-    SC_CUDA(cudaMemcpyAsync(ln.kval.p, k_all.data(), k_all.size() * sizeof(double),
-                            cudaMemcpyHostToDevice, ln.stream), "upload wavenumbers");
+                            cudaMemcpyHostToDevice, ln.stream), "upload amplitudes and wavenumbers");
     std::vector<Chunk> ch;
     int first_cls = -1, first_splits = -1;
     for (int r = 0; r < n_req; ++r) {
         const sc_request& q = reqs[r];
         st = plan_request(ctx, ln, tabs[r], q.omegas, q.n_omega, dom[r], q.points_xyz, q.n_points,
-                          (const double*)ln.amp.p + amp_off[r], (const double*)ln.kval.p + om_off[r],
+                          (const double*)ln.amp.p + amp_off[r], (const double*)ln.amp.p + n_amp + om_off[r],
                           (float2*)q.E_out, (float2*)q.B_out, ch);
         if (st != SC_OK) return st;
         if (r == 0 && !ch.empty()) {
@@ -851,8 +850,9 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     sc_status st;
     std::vector<double> kv(n_omega);
     for (int i = 0; i < n_omega; ++i) kv[i] = 2.0 * kPi * omegas[i];
+    const double dk_rot = rotation_step(kv);
+    kv.insert(kv.end(), times, times + n_t);  // wavenumbers, then times, one upload
     if ((st = ensure(ctx, ctx->tkval, kv.size() * sizeof(double))) != SC_OK) return st;
-    if ((st = ensure(ctx, ctx->tvals, (size_t)n_t * sizeof(double))) != SC_OK) return st;
     const bool tensor = sc::idft_on_tensor(n_omega, n_t);
     if ((st = ensure(ctx, ctx->phasor, tensor ? sc::idft_scratch_bytes(n_omega, n_vals, n_t)
                                               : (size_t)n_omega * n_t * sizeof(float2))) != SC_OK) return st;
@@ -875,19 +875,19 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
         dEt = (float*)ctx->tE.p;
         dBt = B_t ? (float*)ctx->tB.p : nullptr;
     }
-    SC_CUDA(cudaMemcpyAsync(ctx->tkval.p, kv.data(), kv.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->stream), "upload wavenumbers");
-    SC_CUDA(cudaMemcpyAsync(ctx->tvals.p, times, (size_t)n_t * sizeof(double), cudaMemcpyHostToDevice, ctx->stream), "upload times");
+    SC_CUDA(cudaMemcpyAsync(ctx->tkval.p, kv.data(), kv.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->stream),
+            "upload wavenumbers and times");
     sc::IdftLaunch l;
     l.f64 = prec == SC_FP64;
     l.n_omega = n_omega;
     l.n_vals = n_vals;
     l.kval = (const double*)ctx->tkval.p;
-    l.t = (const double*)ctx->tvals.p;
+    l.t = l.kval + n_omega;
     l.n_t = n_t;
     l.dk = dk;
     l.phasor = (float2*)ctx->phasor.p;
     l.table = (unsigned char*)ctx->phasor.p;
-    l.dk_rot = rotation_step(kv);
+    l.dk_rot = dk_rot;
     l.err = ctx->d_err;
     l.accumulate = accumulate;
     for (int pass = 0; pass < (B_spec && !tensor ? 2 : 1); ++pass) {

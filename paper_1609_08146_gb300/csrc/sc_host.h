@@ -134,7 +134,7 @@ struct sc_ctx {
     std::string err = "no error";
     std::list<sch::Table> tables;
     uint64_t tick = 0;
-    sch::DevBuf pts, outE, outB, tkval, tvals, phasor, specE, specB, tE, tB;
+    sch::DevBuf pts, outE, outB, tkval, phasor, specE, specB, tE, tB;
     sch::DevBuf fpts, fspecE, fspecB, ftE, ftB;  // sc_eval_time_domain: points, chunk spectra, E(t), B(t)
     double2* d_trig = nullptr;     // sine and cosine table of the FP64 field sum
     int* d_err = nullptr;
@@ -159,6 +159,9 @@ struct sc_ctx {
     int mfie_order = 0;             // 1: add the first MFIE correction (sc_eval)
     int mfie_rho = 64, mfie_phi = 128;  // its polar rule about each node
     sch::DevBuf mfie_geo, mfie_zern, mfie_gl, mfie_dJ;
+    // points per item and resident CTAs of each kernel class, once asked for (the
+    // occupancy query takes a microsecond)
+    int shape_ppc[sc::kNumClasses] = {}, shape_slots[sc::kNumClasses] = {};
     uint64_t graph_tick = 0;
     uint64_t graph_captures = 0, graph_replays = 0;
     std::map<std::tuple<int, int, int, int, int, int>, int> tuned;  // shape -> split count
