@@ -586,6 +586,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         const unsigned mine = warp == 8;
         constexpr unsigned kAll = 0xffffffffu;
         const uint64_t ah0 = stage_desc(smem_u32(smem));
+        const bool leader = elect_one();
         unsigned fb = 0;  // run number: accumulator fb & 1, its stages' phase fb >> 1
         bool go = true;
         for (long long item = blockIdx.x; item < b.n_items && go; item += gridDim.x) {
@@ -599,6 +600,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 // the accumulator's last run has been read (the first two waits pass at once)
                 go = __all_sync(kAll, field_wait(&accempty[buf], use ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE);
                 if (!go) break;
+                tc_fence_after();
                 const uint32_t d = tmem + buf * L::DCOLS;
                 const uint64_t ab = ah0 + buf * (kFoldTiles * (L::STAGE >> 4));
                 uint64_t* fullb = full + buf * kFoldTiles;
@@ -612,10 +614,9 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                                         field_wait(&fullb[i], use, s_abort, b.abort, timed_out) == WAIT_DONE);
                     if (!go) break;
                     if (i + 1 < kFoldTiles) ready = mbar_test(&fullb[i + 1], use);  // asked for ahead
-                    tc_fence_after();
                     const uint64_t ah = ab + i * (L::STAGE >> 4);
                     const uint64_t al = ah + (kABytes >> 4), bh = ah + (2 * kABytes >> 4);
-                    if (elect_one()) {
+                    if (leader) {
                         if (i < cnt) {
                             mma_f16(d, ah, bh, stage_idesc(2 * L::NP), i > 0);            // hi (hi | lo)
                             mma_f16(d + L::NP, al, bh, stage_idesc(L::NC), 1);            // lo hi
@@ -625,12 +626,11 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                         mma_commit(&emptyb[i]);
                         if (i + 1 == kFoldTiles) mma_commit(&accfull[buf]);
                     }
-                    __syncwarp();
                 }
             }
         }
         // no MMA may be in flight when the tensor memory is freed
-        if (elect_one()) mma_commit(&drain[mine]);
+        if (leader) mma_commit(&drain[mine]);
         __syncwarp();
         if (mbar_wait(&drain[mine], 0) != WAIT_DONE) timed_out = true;
     } else if (prod_index(warp) < kProd) {
