@@ -400,7 +400,7 @@ void class_layout(int cls, int* tpp, int* opt)
         {8, 5}, {8, 6}, {8, 7}, {8, 8}, {16, 8}, {32, 8},                   // 15..20
         {64, 8}, {128, 8}, {256, 8},                                        // 21..23 grouped
         {1, 8}, {4, 3}, {4, 4}, {16, 3}, {16, 4}, {32, 4},                  // 24..29
-        {64, 2}, {64, 4}};                                                  // 30, 31 tensor (rows)
+        {32, 2}, {32, 4}, {64, 4}};                                         // 30..32 tensor (rows)
     const int c = cls < 0 || cls >= kNumClasses ? 0 : cls;
     *tpp = kLayout[c][0];
     *opt = kLayout[c][1];

@@ -11,12 +11,12 @@
 // theta_{n2} = 2 pi delta_{n2} Phi, with the offsets delta symmetric about
 // zero, so that +delta and -delta share their cosine and sine columns:
 //     D[row, col] = sum_j A[row, j] B[col, j]
-//   rows  64 row phasors, cosine and sine (M = 128),
+//   rows  R row phasors, cosine and sine (M = 2 R = 64 or 128),
 //   cols  12 coefficients times N2 trigonometric columns (N = 12 N2),
 //   K     the nodes.
 // N2 omegas per row phasor come out of 12 N2 real columns: no product is
-// computed twice, and a pair costs 128 + 12 N2 operand values instead of the
-// direct kernel's 24 FP32 operations for each of its 64 N2 omegas.
+// computed twice, and a pair costs 2 R + 12 N2 operand values instead of the
+// direct kernel's 24 FP32 operations for each of its R N2 omegas.
 //
 // Precision.  Every operand value x is split into two halves, hi = fp16(x) and
 // lo = fp16(x - hi), 22 bits in all, and three products are accumulated: hi hi
@@ -38,12 +38,16 @@
 // evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
 // Shared memory is busy 72% of the time, half by the operands' stores and half
 // by the MMAs' reads of them, the schedulers issue in 60% of the cycles, and
-// the tensor pipe works 26%.  A pair's cost is mostly its 128 row values and
-// depends little on N2, so the rate falls in proportion to the omega count:
-// 2.95e12 at 128 omegas, 1.6e12 at 48, 1.1e12 at 32 (direct: 1.14, 1.04,
-// 1.00e12); the lines between the classes lie where the measured rates cross:
-// from 25 omegas the tensor kernel (24: direct 0.98, tensor 0.85e12; 26: 0.83,
-// 0.91), 4 omegas per row phasor above 128.
+// the tensor pipe works 26%.  At a few dozen omegas a tile's fixed work (the
+// pair's geometry, three rotations, barriers) counts for most of it.
+//
+// Where the lines between the classes lie (256^2 nodes, 4160 points, 1e11
+// evaluations a second): 24 omegas, direct 9.8, here 8.5; 25: 8.3 and 10.5; 48:
+// 10.4 and 17.4.  32 row phasors of 2 omegas up to 64 omegas (25: 10.5 against 9.5
+// with 64 rows, whose reads of shared memory M = 64 halves; 64: 21.1 against 21.5),
+// of 4 up to 128 (128: 33.9 against 30.7 on 64 rows of 2, with a quarter fewer
+// operand values; 100: 26.5, 25.5), 64 rows of 4 above (256: 43.1; rows of 3 from
+// 129 to 192 gained nothing).
 //
 // Structure (one CTA per SM, 16 warps; shared memory holds ten stages):
 //   warps 0-3   read a finished accumulator (TMEM, two of them), keep the
@@ -71,7 +75,6 @@ namespace sc {
 
 namespace {
 
-constexpr int kRows = 64;                   // row phasors (cosine and sine: M = 128)
 constexpr int kFoldTiles = 5;               // node tiles per run of an accumulator
 constexpr int kStages = 2 * kFoldTiles;     // operand stages (one node tile each): half for either accumulator
 constexpr int kProd = kStages;              // producer warps, each with a stage of its own
@@ -82,16 +85,17 @@ static_assert(4 + 2 + kProd <= kTensorThreads / 32, "warps");
 constexpr int kEpiRegs = 176, kOtherRegs = 112;
 static_assert(128 * kEpiRegs + 384 * kOtherRegs <= 65536, "register split");
 constexpr int kBlkBytes = kTile * 16;           // a block of 8 rows (or columns) of a stage's 32 nodes
-constexpr int kABytes = 2 * kRows / 8 * kBlkBytes;  // one half (hi or lo) of A
 
-template <int N2>
+// N2 omegas per row phasor, R row phasors (M = 2 R rows of A)
+template <int N2, int R>
 struct Tens {
+    static constexpr int ABYTES = 2 * R / 8 * kBlkBytes;  // one half (hi or lo) of A
     static constexpr int N = 12 * N2;
     static constexpr int NP = (N + 7) / 8 * 8;     // rounded to core matrices
-    static constexpr int NC = (NP + 15) / 16 * 16; // the lo x hi product's columns (M = 128 wants 16s)
+    static constexpr int NC = R == 64 ? (NP + 15) / 16 * 16 : NP;  // the lo x hi product (M = 128 wants 16s)
     static constexpr int DCOLS = NP + NC;          // one accumulator: NP hi hi, then hi lo + lo hi
     static constexpr int ALLOC = DCOLS <= 32 ? 64 : (DCOLS <= 64 ? 128 : (DCOLS <= 128 ? 256 : 512));
-    static constexpr int STAGE = 2 * kABytes + 2 * (NP / 8) * kBlkBytes;
+    static constexpr int STAGE = 2 * ABYTES + 2 * (NP / 8) * kBlkBytes;
     static constexpr int OFF_BAR = kStages * STAGE;
     static constexpr int SMEM = OFF_BAR + 256;
     static_assert(2 * NP % 16 == 0, "hi product width");
@@ -102,8 +106,6 @@ struct Tens {
 // Stage layout, MN-major: 128 bytes from one block of 8 nodes to the next,
 // kBlkBytes from one block of 8 rows or columns to the next.
 __device__ __forceinline__ uint64_t stage_desc(uint32_t addr) { return smem_desc(addr, 128, kBlkBytes); }
-
-__host__ __device__ constexpr uint32_t stage_idesc(int n) { return mma_idesc(2 * kRows, n, true, true); }
 
 // Segments of eight row phasors that n_omega omegas take, and the one the
 // seeds start from (then outwards both ways).
@@ -178,6 +180,7 @@ __device__ __forceinline__ bool launch_aborted(const BatchLaunch& b, volatile in
 // n (n + 1) / 2, is multiplied by 6 and not by the 21 of a chain from one end.
 // Steps alternate -c, -c, +c, which saves the negation; slots 1, 2, 5, 6 come
 // out negated and the epilogue turns them back.
+template <int ABYTES>
 __device__ __forceinline__ void store_segment(unsigned char* a_hi, float2 seed, float2 rot, float2 cc, float2 ncc)
 {
     float2 ph[8];
@@ -192,27 +195,27 @@ __device__ __forceinline__ void store_segment(unsigned char* a_hi, float2 seed, 
                          make_float2(ph[4].x, ph[5].x), make_float2(ph[6].x, ph[7].x)};
     const float2 d[4] = {make_float2(ph[0].y, ph[1].y), make_float2(ph[2].y, ph[3].y),
                          make_float2(ph[4].y, ph[5].y), make_float2(ph[6].y, ph[7].y)};
-    split_store8(a_hi, a_hi + kABytes, c);
-    split_store8(a_hi + kBlkBytes, a_hi + kABytes + kBlkBytes, d);
+    split_store8(a_hi, a_hi + ABYTES, c);
+    split_store8(a_hi + kBlkBytes, a_hi + ABYTES + kBlkBytes, d);
 }
 
 // One tile's operands; `wait` (bounded) blocks until the MMAs have read the
 // stage's last contents and is placed after everything that can be computed
 // without the stage.  False: aborted or expired.
-template <int N2, typename Wait>
+template <int N2, int R, typename Wait>
 __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float nd[9], const TItem& it, int lane,
                                              int nseg, const TensorSteps& w, Wait wait)
 {
-    using L = Tens<N2>;
+    using L = Tens<N2, R>;
     const float px = nd[0], py = nd[1], pz = nd[2], pn = nd[3], wo = nd[4];
     const float4 P = it.P;
     // pair geometry and phase as in pair_coefs()
     const float dx = px - P.x, dy = py - P.y, dz = pz - P.z;
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
     const float ir = rsqrtf(r2);
-    const float R = r2 * ir;
+    const float dist = r2 * ir;
     const float D = fmaf(-2.0f * P.x, px, fmaf(-2.0f * P.y, py, fmaf(-2.0f * P.z, pz, P.w)));
-    const float phi = __fdividef(D, R + pn) + wo;
+    const float phi = __fdividef(D, dist + pn) + wo;
     const float rx = dx * ir, ry = dy * ir, rz = dz * ir;
     const float sir = it.js * ir;
     const float ux = nd[5] * sir, uy = nd[6] * sir, uz = nd[7] * sir;
@@ -247,7 +250,7 @@ __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float n
     float2 up = phasor_2wphi_mufu(w.seed.x, w.seed.y, phi);
     if (!wait()) return false;
 
-    unsigned char* b_hi = stage + 2 * kABytes + lane * 16;
+    unsigned char* b_hi = stage + 2 * L::ABYTES + lane * 16;
     unsigned char* b_lo = b_hi + (L::NP / 8) * kBlkBytes;
 #pragma unroll
     for (int blk = 0; blk < L::NP / 8; ++blk) {
@@ -268,18 +271,18 @@ __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float n
     const int s0 = seed_seg(nseg);
     unsigned char* a_up = stage + lane * 16 + 2 * s0 * kBlkBytes;
     unsigned char* a_dn = a_up - 2 * kBlkBytes;
-    store_segment(a_up, up, rot, cc, ncc);
+    store_segment<L::ABYTES>(a_up, up, rot, cc, ncc);
     const int both = nseg - 1 - s0;  // segments on either side (an even count has one more below)
 #pragma unroll 1
     for (int s = 0; s < both; ++s) {
         up = cmul(up, rseg);
         a_up += 2 * kBlkBytes;
-        store_segment(a_dn, dn, rot, cc, ncc);
-        store_segment(a_up, up, rot, cc, ncc);
+        store_segment<L::ABYTES>(a_dn, dn, rot, cc, ncc);
+        store_segment<L::ABYTES>(a_up, up, rot, cc, ncc);
         a_dn -= 2 * kBlkBytes;
         dn = cmul(dn, rback);
     }
-    if (s0 > both) store_segment(a_dn, dn, rot, cc, ncc);
+    if (s0 > both) store_segment<L::ABYTES>(a_dn, dn, rot, cc, ncc);
     return true;
 }
 
@@ -309,7 +312,8 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float v)
 // ^ 8) imaginary ones, Im E = k Re S1 - Im S2: either needs the partner's cosine
 // column of S1 and sine column of S2, one exchange each.
 template <int N2>
-__device__ __forceinline__ void write_item(const TItem& it, int row, const float2* s2, const float2* e2)
+__device__ __forceinline__ void write_item(const TItem& it, int row, bool own_row, const float2* s2,
+                                           const float2* e2)
 {
     const FieldLaunch& p = *it.f;
     const int seg = row >> 4, idx = row & 7;
@@ -364,7 +368,7 @@ __device__ __forceinline__ void write_item(const TItem& it, int row, const float
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (!(zero && h == 1) && nn[h] < p.n_omega)
+            if (!(zero && h == 1) && own_row && nn[h] < p.n_omega)
 #pragma unroll
                 for (int c = 0; c < 6; ++c) base[(size_t)nn[h] * kAcc + 2 * c] = dst_v[h][c];
     }
@@ -391,12 +395,12 @@ struct ProdSync {
     }
 };
 
-template <int N2>
+template <int N2, int R>
 __device__ __noinline__ bool plain_item(unsigned char* smem, const TItem& it, int w, int lane, ProdSync& ps)
 {
-    constexpr int NB = kRows * N2 / 32;  // omegas per lane
-    using L = Tens<N2>;
-    static_assert(L::STAGE >= kRows * N2 * 12 * 4 && L::STAGE >= 32 * 16 * 4, "stage too small for the plain loop");
+    constexpr int NB = R * N2 / 32;  // omegas per lane
+    using L = Tens<N2, R>;
+    static_assert(L::STAGE >= R * N2 * 12 * 4 && L::STAGE >= 32 * 16 * 4, "stage too small for the plain loop");
     const FieldLaunch& p = *it.f;
     float* rows = reinterpret_cast<float*>(smem + w * L::STAGE);
     const double om0 = (double)p.om_hi0 + (double)p.om_lo0, dom = (double)p.dom_hi + (double)p.dom_lo;
@@ -479,10 +483,10 @@ __device__ __forceinline__ int prod_index(int warp)
     return (warp & 3) ? 3 * ((warp >> 2) - 1) + (warp & 3) - 1 : 9;
 }
 
-template <int N2>
+template <int N2, int R>
 __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const __grid_constant__ BatchLaunch b)
 {
-    using L = Tens<N2>;
+    using L = Tens<N2, R>;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);  // [kStages] stage written
     uint64_t* empty = full + kStages;                                 // [kStages] stage read by the MMAs
@@ -524,7 +528,9 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
     if (warp < 4) {
         // ---------------- epilogue ----------------
-        const int row = warp * 32 + lane;
+        // M = 128: lane = row; M = 64: 16 rows in the first half of every warp's lanes
+        const int row = R == 64 ? warp * 32 + lane : warp * 16 + (lane & 15);
+        const bool own_row = R == 64 || lane < 16;
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
         long long fb = 0;
         bool stop = false;
@@ -572,7 +578,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&accempty[buf]);
             }
-            if (!stop) write_item<N2>(it, row, s, e);
+            if (!stop) write_item<N2>(it, row, own_row, s, e);
         }
     } else if (warp == 4 || warp == 8) {
         // ---------------- MMA issue ----------------
@@ -615,13 +621,13 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                     if (!go) break;
                     if (i + 1 < kFoldTiles) ready = mbar_test(&fullb[i + 1], use);  // asked for ahead
                     const uint64_t ah = ab + i * (L::STAGE >> 4);
-                    const uint64_t al = ah + (kABytes >> 4), bh = ah + (2 * kABytes >> 4);
+                    const uint64_t al = ah + (L::ABYTES >> 4), bh = ah + (2 * L::ABYTES >> 4);
                     if (leader) {
                         if (i < cnt) {
-                            mma_f16(d, ah, bh, stage_idesc(2 * L::NP), i > 0);            // hi (hi | lo)
-                            mma_f16(d + L::NP, al, bh, stage_idesc(L::NC), 1);            // lo hi
-                            mma_f16(d, ah + 16, bh + 16, stage_idesc(2 * L::NP), 1);      // nodes 16..31
-                            mma_f16(d + L::NP, al + 16, bh + 16, stage_idesc(L::NC), 1);
+                            mma_f16(d, ah, bh, mma_idesc(2 * R, 2 * L::NP, true, true), i > 0);            // hi (hi | lo)
+                            mma_f16(d + L::NP, al, bh, mma_idesc(2 * R, L::NC, true, true), 1);            // lo hi
+                            mma_f16(d, ah + 16, bh + 16, mma_idesc(2 * R, 2 * L::NP, true, true), 1);      // nodes 16..31
+                            mma_f16(d + L::NP, al + 16, bh + 16, mma_idesc(2 * R, L::NC, true, true), 1);
                         }
                         mma_commit(&emptyb[i]);
                         if (i + 1 == kFoldTiles) mma_commit(&accfull[buf]);
@@ -650,7 +656,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
                 if (fb0 > half && field_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out) != WAIT_DONE)
                     break;
-                if (!plain_item<N2>(smem, it, w, lane, ps)) break;
+                if (!plain_item<N2, R>(smem, it, w, lane, ps)) break;
                 continue;
             }
             const int nseg = segments(it.f->n_omega, N2);
@@ -678,7 +684,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 auto stage_free = [&] {
                     return field_wait(&empty[w], use ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE;
                 };
-                if (!(tr >= 0 ? produce_tile<N2>(smem + w * L::STAGE, cur, it, lane, nseg, steps, stage_free)
+                if (!(tr >= 0 ? produce_tile<N2, R>(smem + w * L::STAGE, cur, it, lane, nseg, steps, stage_free)
                               : stage_free())) {
                     stop = true;
                     break;
@@ -706,11 +712,11 @@ float2 ff(double w)
     return make_float2(hi, (float)(w - (double)hi));
 }
 
-template <int N2>
+template <int N2, int R>
 int launch_tensor(const BatchLaunch& b, int grid, cudaStream_t s)
 {
-    using L = Tens<N2>;
-    auto kern = field_tensor_kernel<N2>;
+    using L = Tens<N2, R>;
+    auto kern = field_tensor_kernel<N2, R>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM);
     if (e != cudaSuccess) return -(int)e;
     kern<<<grid, kTensorThreads, L::SMEM, s>>>(b);
@@ -720,15 +726,18 @@ int launch_tensor(const BatchLaunch& b, int grid, cudaStream_t s)
 
 }  // namespace
 
+// Classes: 2 omegas on each of 32 row phasors, 4 on 32, 4 on 64.
+static int class_n2(int cls) { return cls == kFirstTensorClass ? 2 : 4; }
+
 int tensor_class(int n_omega)
 {
     if (n_omega < kTensorMinOmega || n_omega > kTensorMaxOmega) return -1;
-    return n_omega <= 2 * kRows ? kFirstTensorClass : kFirstTensorClass + 1;
+    return kFirstTensorClass + (n_omega <= 64 ? 0 : (n_omega <= 128 ? 1 : 2));
 }
 
 void tensor_prepare(int cls, FieldLaunch& f)
 {
-    const int n2 = cls == kFirstTensorClass ? 2 : 4;
+    const int n2 = class_n2(cls);
     const double om0 = (double)f.om_hi0 + (double)f.om_lo0, dom = (double)f.dom_hi + (double)f.dom_lo;
     const double seed_row = 8 * seed_seg(segments(f.n_omega, n2)) + 3;
     f.steps.seed = ff(om0 + (seed_row * n2 + 0.5 * (n2 - 1)) * dom);
@@ -742,14 +751,20 @@ void tensor_prepare(int cls, FieldLaunch& f)
 void tensor_field_shape(int cls, int device, int* ppc, int* slots)
 {
     *ppc = 1;
-    *slots = cls == kFirstTensorClass
-                 ? resident(field_tensor_kernel<2>, kTensorThreads, Tens<2>::SMEM, device)
-                 : resident(field_tensor_kernel<4>, kTensorThreads, Tens<4>::SMEM, device);
+    switch (cls - kFirstTensorClass) {
+    case 0: *slots = resident(field_tensor_kernel<2, 32>, kTensorThreads, Tens<2, 32>::SMEM, device); break;
+    case 1: *slots = resident(field_tensor_kernel<4, 32>, kTensorThreads, Tens<4, 32>::SMEM, device); break;
+    default: *slots = resident(field_tensor_kernel<4, 64>, kTensorThreads, Tens<4, 64>::SMEM, device);
+    }
 }
 
 int launch_tensor_field(int cls, const BatchLaunch& b, int grid, cudaStream_t s)
 {
-    return cls == kFirstTensorClass ? launch_tensor<2>(b, grid, s) : launch_tensor<4>(b, grid, s);
+    switch (cls - kFirstTensorClass) {
+    case 0: return launch_tensor<2, 32>(b, grid, s);
+    case 1: return launch_tensor<4, 32>(b, grid, s);
+    default: return launch_tensor<4, 64>(b, grid, s);
+    }
 }
 
 }  // namespace sc

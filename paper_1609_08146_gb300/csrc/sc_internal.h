@@ -100,9 +100,10 @@ struct BatchLaunch {
 // Kernel class for a chunk of n_omega (<= 2048) omegas: 0..20 the direct
 // kernel (1 to 32 threads per point, 1..8 omegas per thread, up to 256
 // omegas), 21..23 the grouped kernel with 64, 128, 256 threads per point,
-// 24..29 alternative direct layouts for the autotuner, 30, 31 the tensor
-// kernel with 2 and 4 omegas per row phasor (up to 128 and 256 omegas).
-constexpr int kNumClasses = 32;
+// 24..29 alternative direct layouts for the autotuner, 30..32 the tensor
+// kernel with 32 row phasors of 2 and of 4 omegas and 64 of 4 (up to 64, 128 and
+// 256 omegas).
+constexpr int kNumClasses = 33;
 constexpr int kFirstGroupedClass = 21;  // grouped classes 21..23
 constexpr int kFirstAltClass = 24;      // alternative direct layouts 24..29 (alt_field_class)
 constexpr int kFirstTensorClass = 30;
