@@ -14,12 +14,14 @@ Metric: obs x node x omega evaluations per second (surface nodes), whole job.
   e2e     the same step through the C-ABI with host buffers: points from
           pinned host memory in, time-domain E(t), B(t) back to pinned host
           memory, copies inside the timed region.
-  roofline  the dominant kernel (FP32 field sum) against the FP32-pipe peak
-          SMs x 128 lanes x clock, counting the algorithmic work of one
-          evaluation of the factorised summand as 28 FP32 instructions (a
-          complex rotation and 12 real coefficients times a complex phasor);
-          the kernel's own form needs 24, and the line reports that
-          fraction too.
+  roofline  the dominant kernel (the field sum on the tensor cores): the
+          tensor operations it executes per evaluation (three fp16 products of
+          split operands, 144) against the measured cuBLAS bf16 rate, and the
+          same throughput against the FP32-pipe peak SMs x 128 lanes x clock,
+          counting the algorithmic work of one evaluation as 28 FP32
+          instructions (a complex rotation and 12 real coefficients times a
+          complex phasor), which is above 1: no FP32 form can reach it.  The
+          8-omega workload, on the FP32 pipe, is reported against that alone.
   cpu_baseline  the FP64 oracle on the host cores over a bounded sample of
           the same workload.
 --impl reference times that oracle as the reference arm.
@@ -45,11 +47,13 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 OPS_PER_EVAL = 28     # algorithmic FP32 instructions per (point, node, omega) of the factorised summand
-KERNEL_OPS_PER_EVAL = 24  # what the kernel issues: three-term phasor recurrence, packed FMAs
-FIELD_KERNEL = "field_direct_kernel<8, 32>"  # 256 omegas: 32 threads of 8 omegas per point
-PROFILE_JSON = os.path.join(ROOT, "profiles", "field_direct_broadband.json")
+KERNEL_OPS_PER_EVAL = 24  # what the direct kernel issues: three-term phasor recurrence, packed FMAs
+# the tensor kernel's operations per evaluation at 256 omegas: 3 products of 128 rows x 48 columns a pair
+TENSOR_OPS_PER_EVAL = 3 * 2 * 128 * 48 / 256
+FIELD_KERNEL = "field_tensor_kernel<4, 64>"  # 256 omegas: 64 row phasors of 4 omegas
+PROFILE_JSON = os.path.join(ROOT, "profiles", "field_tensor_broadband.json")
 CSRC = os.path.join(ROOT, "paper_1609_08146_gb300", "csrc")
-FIELD_SRCS = [os.path.join(CSRC, f) for f in ("sc_field_direct.cu", "sc_field_common.cuh")]
+FIELD_SRCS = [os.path.join(CSRC, f) for f in ("sc_field_tensor.cu", "sc_tensor.cuh", "sc_field_common.cuh")]
 
 
 def parse():
@@ -697,19 +701,31 @@ def main():
     max_mhz = clk.get("sm_max_mhz") or 2070.0
     peak = sms * 128 * max_mhz * 1e6 * 1e-12  # TOP/s of FP32 lane-ops at the maximum SM clock
     achieved = field_evals * OPS_PER_EVAL / (field_ms / 1000.0) * 1e-12
-    roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TOP/s",
-            "frac": achieved / peak,
-            "traffic": profile_traffic() if args.workload != "small_omega" else None,
-            "kernel": FIELD_KERNEL if args.workload != "small_omega" else "field_direct_kernel<4, 2>",
+    fp32 = {"achieved": achieved, "peak": peak, "unit": "TOP/s", "frac": achieved / peak,
             "ops_per_eval": OPS_PER_EVAL,
             "ops_basis": "algorithmic work per evaluation: complex rotation (4) + 12 real coefficients "
                          "x complex phasor (24)",
-            "kernel_ops_per_eval": KERNEL_OPS_PER_EVAL,
-            "frac_at_kernel_ops": achieved / peak * KERNEL_OPS_PER_EVAL / OPS_PER_EVAL,
-            "peak_basis": "%d SMs x 128 FP32 lanes x %.0f MHz (max SM clock)" % (sms, max_mhz),
-            "kernel_ms": field_ms}
+            "peak_basis": "%d SMs x 128 FP32 lanes x %.0f MHz (max SM clock)" % (sms, max_mhz)}
+    if args.workload == "small_omega":
+        roof = fp32
+        roof.update(bound="alu", kernel="field_direct_kernel<4, 2>", traffic=None,
+                    kernel_ops_per_eval=KERNEL_OPS_PER_EVAL,
+                    frac_at_kernel_ops=achieved / peak * KERNEL_OPS_PER_EVAL / OPS_PER_EVAL)
+    else:
+        try:
+            tpeak = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["bf16_tflops"]
+            tbasis = "measured cuBLAS bf16 GEMM"
+        except (OSError, ValueError, KeyError):
+            tpeak, tbasis = 1900.0, "fallback: an earlier cuBLAS bf16 measurement"
+        tops = field_evals * TENSOR_OPS_PER_EVAL / (field_ms / 1000.0) * 1e-12
+        roof = {"bound": "shared memory (operand stores and reads)", "achieved": tops, "peak": tpeak,
+                "unit": "TFLOP/s", "frac": tops / tpeak, "peak_basis": tbasis, "traffic": profile_traffic(),
+                "kernel": FIELD_KERNEL, "ops_per_eval": TENSOR_OPS_PER_EVAL,
+                "ops_basis": "fp16 tensor operations executed: three products of split operands",
+                "fp32_pipe_equivalent": fp32}
+    roof["kernel_ms"] = field_ms
     if clk.get("sm_mhz"):
-        roof["frac_at_sampled_clock"] = achieved / (sms * 128 * clk["sm_mhz"] * 1e6 * 1e-12)
+        fp32["frac_at_sampled_clock"] = achieved / (sms * 128 * clk["sm_mhz"] * 1e6 * 1e-12)
     # what the FMA and MUFU pipes sustain on pure instruction streams (after the timed region)
     probes = ctx.measure_alu_peaks()
     fma_t = probes["fp32_lane_ops_per_s"] * 1e-12
@@ -720,7 +736,7 @@ def main():
         "fma_frac_of_peak": max(fma_t, fma2_t) / peak,
         "basis": "sc_measure_alu_peaks: independent FFMA, FFMA2 and MUFU rsqrt streams on every SM, "
                  "best of 3 launches, clocks not pinned"}
-    roof["frac_of_measured_fma"] = achieved / max(fma_t, fma2_t)
+    fp32["frac_of_measured_fma"] = achieved / max(fma_t, fma2_t)
 
     # ---- plain FP64 GPU form of the same sum, on a point subsample
     sub = torch.tensor(w["points"][::65], device=dev)  # 64 points
