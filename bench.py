@@ -786,7 +786,7 @@ def main():
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": w["name"], "mirror_nodes": n_nodes, "points": npts,
                        "omegas": len(om), "time_samples": len(times), "f_lambda0": mc["f"],
-                       "precision": "FP32 compensated phase, FP64 cross-split reduction",
+                       "precision": "FP32 compensated phase, split-operand tensor products, compensated sums, FP64 epilogue",
                        "l2": "256 MB memset between steps, outside the timed events",
                        "parallelism": ("points sharded over %d GPUs" % world if strong else
                                        "replicas" if world > 1 else "single GPU")},
