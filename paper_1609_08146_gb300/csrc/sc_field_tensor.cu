@@ -34,19 +34,24 @@
 // norms over sizes and beams at random: 1.9e-7 to 4.1e-7 here, 2.8e-7 to
 // 1.1e-6 with the FP32 kernels.
 //
-// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 63 ms, 4.4e12
+// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 62.5 ms, 4.5e12
 // evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
 // Shared memory is busy 72% of the time, half by the operands' stores and half
 // by the MMAs' reads of them, the schedulers issue in 60% of the cycles, and
 // the tensor pipe works 26%.  At a few dozen omegas a tile's fixed work (the
-// pair's geometry, three rotations, barriers) counts for most of it.
+// pair's geometry, three rotations, barriers) counts for most of it: at 32
+// omegas shared memory is busy 80%, the schedulers issue in 69% of the cycles, and
+// the producers wait for a stage a fifth of their time.  No one of them binds
+// alone there: twenty stages (a producer then need not wait), four accumulators,
+// and the halves of A stacked into one M = 128 MMA (fewer MMAs and reads) each
+// changed the time by less than 2%, both ways.
 //
 // Where the lines between the classes lie (256^2 nodes, 4160 points, 1e11
 // evaluations a second): 24 omegas, direct 9.8, here 8.5; 25: 8.3 and 10.5; 48:
-// 10.4 and 17.4.  32 row phasors of 2 omegas up to 64 omegas (25: 10.5 against 9.5
+// 10.4 and 17.5.  32 row phasors of 2 omegas up to 64 omegas (25: 10.5 against 9.5
 // with 64 rows, whose reads of shared memory M = 64 halves; 64: 21.1 against 21.5),
 // of 4 up to 128 (128: 33.9 against 30.7 on 64 rows of 2, with a quarter fewer
-// operand values; 100: 26.5, 25.5), 64 rows of 4 above (256: 43.1; rows of 3 from
+// operand values; 100: 26.5, 25.5), 64 rows of 4 above (256: 43.6; rows of 3 from
 // 129 to 192 gained nothing).
 //
 // Structure (one CTA per SM, 16 warps; shared memory holds ten stages):
@@ -174,6 +179,38 @@ __device__ __forceinline__ bool launch_aborted(const BatchLaunch& b, volatile in
 // ------------------------------------------------------------------------
 // Producers
 
+// The rotations: phasor_2wphi() with the sine and cosine of its reduced argument
+// evaluated here, with one range reduction instead of two: 128 omegas 10.33 ->
+// 10.13 ms, 192: 14.79 -> 14.46, 256: 16.25 -> 16.00 (256^2 nodes, 4160 points),
+// 25 to 64 as before.  The quarter turn is taken off by
+// adding and subtracting 1.5 2^23, whose low bits then hold its number, and the
+// residual xl is added after it, where it costs the least rounding.  On |t| <=
+// 1/4, z = t^2,
+//     cos pi t = 1 + z C(z),   sin pi t = pi t + t P(z),
+// with cubics C and P that are minimax fits (Remez exchange, absolute error of
+// the functions 5e-11 and 1.2e-9) rounded to FP32; P's constant carries what FP32
+// pi is off.  Measured over t: 5.7e-8 and 4.0e-8 at most.
+__device__ __forceinline__ float2 rotation_2wphi(float w_hi, float w_lo, float phi)
+{
+    const float a = 2.0f * w_hi;
+    const float xh = a * phi;
+    const float xl = fmaf(2.0f * w_lo, phi, fmaf(a, phi, -xh));
+    const float d = fmaf(-2.0f, rintf(0.5f * xh), xh);
+    const float m = fmaf(d + xl, 2.0f, 12582912.0f);
+    const float t = fmaf(m - 12582912.0f, -0.5f, d) + xl;
+    const float z = t * t;
+    const float2 zz = make_float2(z, z);
+    float2 v = make_float2(0.23142955f, -0.58782387f);
+    v = __ffma2_rn(v, zz, make_float2(-1.3350585f, 2.5496302f));
+    v = __ffma2_rn(v, zz, make_float2(4.0587077f, -5.1677036f));
+    v = __ffma2_rn(v, zz, make_float2(-4.934802f, -1.3038593e-07f));
+    const float c = fmaf(z, v.x, 1.0f), s = fmaf(t, 3.14159274f, t * v.y);
+    const unsigned q = __float_as_uint(m);  // quarter turns, mod 4
+    const float x = (q & 1) ? s : c, y = (q & 1) ? c : s;
+    return make_float2(__uint_as_float(__float_as_uint(x) ^ (((q + 1) & 2) << 30)),
+                       __uint_as_float(__float_as_uint(y) ^ ((q & 2) << 30)));
+}
+
 // One segment: eight row phasors from the seed of its fourth, its neighbour by
 // one rotation, and the three-term recurrence from these two outwards: three
 // steps at most, so that the rounding of c = 2 cos, which n steps multiply by
@@ -233,7 +270,7 @@ __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float n
     // cosines and sines of the column offsets: m steps (odd N2) or m + 1/2 (even)
     float trig[N2];
     {
-        float2 q = N2 > 1 ? phasor_2wphi(w.col.x, w.col.y, phi) : make_float2(1.f, 0.f);
+        float2 q = N2 > 1 ? rotation_2wphi(w.col.x, w.col.y, phi) : make_float2(1.f, 0.f);
         const float2 full = (N2 & 1) ? q : cmul(q, q);
         if (N2 & 1) trig[0] = 1.f;
 #pragma unroll
@@ -245,8 +282,8 @@ __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float n
     }
     // row phasors: one seed (MUFU sine and cosine, as in the direct kernel) and
     // the rotations between rows and between segments
-    const float2 rot = phasor_2wphi(w.row.x, w.row.y, phi);
-    const float2 rseg = phasor_2wphi(w.seg.x, w.seg.y, phi);
+    const float2 rot = rotation_2wphi(w.row.x, w.row.y, phi);
+    const float2 rseg = rotation_2wphi(w.seg.x, w.seg.y, phi);
     float2 up = phasor_2wphi_mufu(w.seed.x, w.seed.y, phi);
     if (!wait()) return false;
 
@@ -656,7 +693,8 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
                 if (fb0 > half && field_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out) != WAIT_DONE)
                     break;
-                if (!plain_item<N2, R>(smem, it, w, lane, ps)) break;
+                const TItem copy = it;  // (a reference to `it` itself would keep it in local memory)
+                if (!plain_item<N2, R>(smem, copy, w, lane, ps)) break;
                 continue;
             }
             const int nseg = segments(it.f->n_omega, N2);
