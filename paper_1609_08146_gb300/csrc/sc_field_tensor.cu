@@ -34,7 +34,7 @@
 // norms over sizes and beams at random: 1.9e-7 to 4.1e-7 here, 2.8e-7 to
 // 1.1e-6 with the FP32 kernels.
 //
-// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 62.5 ms, 4.5e12
+// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 52.2 ms, 5.3e12
 // evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
 // Shared memory is busy 72% of the time, half by the operands' stores and half
 // by the MMAs' reads of them, the schedulers issue in 60% of the cycles, and
@@ -51,7 +51,7 @@
 // 10.4 and 17.5.  32 row phasors of 2 omegas up to 64 omegas (25: 10.5 against 9.5
 // with 64 rows, whose reads of shared memory M = 64 halves; 64: 21.1 against 21.5),
 // of 4 up to 128 (128: 33.9 against 30.7 on 64 rows of 2, with a quarter fewer
-// operand values; 100: 26.5, 25.5), 64 rows of 4 above (256: 43.6; rows of 3 from
+// operand values; 100: 26.5, 25.5), 64 rows of 4 above (256: 52.1; rows of 3 from
 // 129 to 192 gained nothing).
 //
 // Structure (one CTA per SM, 16 warps; shared memory holds ten stages):
@@ -682,19 +682,12 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         const unsigned half = w / kFoldTiles;
         const int slot = w % kFoldTiles;
         unsigned fb0 = 0;     // runs of this CTA's items so far
-        bool stop = false;
-        ProdSync ps{psync, s_abort, b.abort, 0, false};
+        bool stop = false, plain = false;
         for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
             if (*s_abort) break;
             const TItem it = tensor_item(b, item);
             if (!it.ok) {
-                // the MMAs may still read the stage this warp borrows: its last run
-                // was the newest one on its half
-                const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
-                if (fb0 > half && field_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out) != WAIT_DONE)
-                    break;
-                const TItem copy = it;  // (a reference to `it` itself would keep it in local memory)
-                if (!plain_item<N2, R>(smem, copy, w, lane, ps)) break;
+                plain = true;
                 continue;
             }
             const int nseg = segments(it.f->n_omega, N2);
@@ -733,7 +726,24 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             }
             fb0 += nruns;
         }
-        timed_out |= ps.timed_out;
+        // The items left over come last, so that nothing of the loop above lives
+        // across this call: called from there it put 17 loads and 9 stores of local
+        // memory into every tile of 256 omegas (256^2 nodes, 4160 points: 15.98 ms, now
+        // 13.38).
+        if (plain && !stop) {
+            // the MMAs may still read the stage this warp borrows: its last run was
+            // the newest one on its half
+            const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
+            if (fb0 > half && field_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out) != WAIT_DONE)
+                stop = true;
+            ProdSync ps{psync, s_abort, b.abort, 0, false};
+            for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
+                if (*s_abort) break;
+                const TItem it = tensor_item(b, item);
+                if (!it.ok && !plain_item<N2, R>(smem, it, w, lane, ps)) break;
+            }
+            timed_out |= ps.timed_out;
+        }
     }
     if (timed_out) atomicOr(b.err, ERR_TIMEOUT);
     tc_fence_before();
