@@ -36,31 +36,30 @@
 //
 // What bounds it.  256 omegas, 512^2 nodes, 4160 points: 52.2 ms, 5.3e12
 // evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
-// Shared memory is busy 72% of the time, half by the operands' stores and half
-// by the MMAs' reads of them, the schedulers issue in 60% of the cycles, and
-// the tensor pipe works 26%.  At a few dozen omegas a tile's fixed work (the
-// pair's geometry, three rotations, barriers) counts for most of it: at 32
-// omegas shared memory is busy 80%, the schedulers issue in 69% of the cycles, and
-// the producers wait for a stage a fifth of their time.  No one of them binds
-// alone there: twenty stages (a producer then need not wait), four accumulators,
-// and the halves of A stacked into one M = 128 MMA (fewer MMAs and reads) each
-// changed the time by less than 2%, both ways.
+// The schedulers issue in two thirds of the cycles and shared memory is busy about
+// as long (operand stores, and the MMAs' reads of them); the tensor pipe works a
+// third of the time.  At a few dozen omegas a tile's fixed work (the pair's
+// geometry, three rotations, barriers) counts for most of it: at 32 omegas shared
+// memory is busy 80%, the schedulers issue in 69% of the cycles, and the producers
+// wait for a stage a fifth of their time.  No one of them binds alone there:
+// twenty stages (a producer then need not wait) and the halves of A stacked into
+// one M = 128 MMA (fewer MMAs and reads) each gained nothing.
 //
 // Where the lines between the classes lie (256^2 nodes, 4160 points, 1e11
-// evaluations a second): 24 omegas, direct 9.8, here 8.5; 25: 8.3 and 10.5; 48:
-// 10.4 and 17.5.  32 row phasors of 2 omegas up to 64 omegas (25: 10.5 against 9.5
+// evaluations a second): 24 omegas, direct 9.8, here 8.5; 25: 8.3 and 10.8; 48:
+// 10.4 and 17.8.  32 row phasors of 2 omegas up to 64 omegas (25: 10.5 against 9.5
 // with 64 rows, whose reads of shared memory M = 64 halves; 64: 21.1 against 21.5),
 // of 4 up to 128 (128: 33.9 against 30.7 on 64 rows of 2, with a quarter fewer
 // operand values; 100: 26.5, 25.5), 64 rows of 4 above (256: 52.1; rows of 3 from
-// 129 to 192 gained nothing).
+// 129 to 192 are no better: 160: 37.3 against 39.6, 192: 42.3 against 44.5).
 //
 // Structure (one CTA per SM, 16 warps; shared memory holds ten stages):
-//   warps 0-3   read a finished accumulator (TMEM, two of them), keep the
+//   warps 0-3   read a finished accumulator (TMEM, two or four), keep the
 //               compensated running sums of the item (one point, one node
 //               split) in registers and write its partials;
-//   warps 4, 8  issue the MMAs, one warp for either accumulator;
+//   warps 4, 8  issue the MMAs, a warp for every second run;
 //   the others  produce operands, each into a stage of its own: lane = node,
-//               five warps per accumulator.  A lane computes its pair's
+//               five warps for every second run.  A lane computes its pair's
 //               geometry, coefficients and phases and writes its operand
 //               columns in the MN-major core-matrix layout (8 rows of one node
 //               are 16 contiguous bytes, so that a warp's stores are
@@ -99,12 +98,16 @@ struct Tens {
     static constexpr int NP = (N + 7) / 8 * 8;     // rounded to core matrices
     static constexpr int NC = R == 64 ? (NP + 15) / 16 * 16 : NP;  // the lo x hi product (M = 128 wants 16s)
     static constexpr int DCOLS = NP + NC;          // one accumulator: NP hi hi, then hi lo + lo hi
-    static constexpr int ALLOC = DCOLS <= 32 ? 64 : (DCOLS <= 64 ? 128 : (DCOLS <= 128 ? 256 : 512));
+    // Accumulators in tensor memory: with four the MMAs need not wait for the
+    // epilogue's last read (25 omegas 6.41 -> 6.23 ms, 64 8.17 -> 7.99); more columns
+    // gain nothing at 256 omegas and cost 2% on small tables.
+    static constexpr int ACCS = N2 <= 2 ? 4 : 2;
+    static constexpr int ALLOC = ACCS * DCOLS <= 64 ? 64 : (ACCS * DCOLS <= 128 ? 128 : (ACCS * DCOLS <= 256 ? 256 : 512));
     static constexpr int STAGE = 2 * ABYTES + 2 * (NP / 8) * kBlkBytes;
     static constexpr int OFF_BAR = kStages * STAGE;
     static constexpr int SMEM = OFF_BAR + 256;
     static_assert(2 * NP % 16 == 0, "hi product width");
-    static_assert(2 * DCOLS <= ALLOC, "tensor memory");
+    static_assert(ACCS * DCOLS <= ALLOC, "tensor memory");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
@@ -527,9 +530,9 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
     extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);  // [kStages] stage written
     uint64_t* empty = full + kStages;                                 // [kStages] stage read by the MMAs
-    uint64_t* accfull = empty + kStages;                                // [2] accumulator finished
-    uint64_t* accempty = accfull + 2;                                 // [2] accumulator read
-    uint64_t* drain = accempty + 2;
+    uint64_t* accfull = empty + kStages;                              // [ACCS] accumulator finished
+    uint64_t* accempty = accfull + L::ACCS;                           // [ACCS] accumulator read
+    uint64_t* drain = accempty + L::ACCS;                             // [2] the MMA warps' last commits
     uint64_t* psync = drain + 2;                                      // the producer warps among themselves
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(psync + 1);
     volatile int* s_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < L::ACCS; ++i) {
             mbar_init(&accfull[i], 1);
             mbar_init(&accempty[i], 4);
         }
@@ -581,8 +584,8 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             for (int c = 0; c < L::N / 2; ++c) s[c] = e[c] = make_float2(0.f, 0.f);
             const float2 neg = make_float2(-1.f, -1.f);
             for (int t = 0; t < it.nt; t += ft, ++fb) {
-                const int buf = (int)(fb & 1);
-                if (field_wait(&accfull[buf], (unsigned)((fb >> 1) & 1), s_abort, b.abort, timed_out) != WAIT_DONE) {
+                const int buf = (int)(fb % L::ACCS);
+                if (field_wait(&accfull[buf], (unsigned)((fb / L::ACCS) & 1), s_abort, b.abort, timed_out) != WAIT_DONE) {
                     stop = true;
                     break;
                 }
@@ -623,14 +626,14 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         // made warp-uniform by a vote or a broadcast, so that descriptors and
         // addresses live in uniform registers, where the MMA takes them from;
         // one elected lane issues.  Issued from a one-lane branch each MMA cost
-        // about 200 cycles.  Two warps, one per accumulator: a tile's barrier,
+        // about 200 cycles.  Two warps, taking turns by runs: a tile's barrier,
         // four MMAs and commit take one warp over 400 cycles, most of them
         // latency, and the producers make a tile in 440.
         const unsigned mine = warp == 8;
         constexpr unsigned kAll = 0xffffffffu;
         const uint64_t ah0 = stage_desc(smem_u32(smem));
         const bool leader = elect_one();
-        unsigned fb = 0;  // run number: accumulator fb & 1, its stages' phase fb >> 1
+        unsigned fb = 0;  // run number: warp and stages fb & 1, accumulator fb % ACCS
         bool go = true;
         for (long long item = blockIdx.x; item < b.n_items && go; item += gridDim.x) {
             if (__any_sync(kAll, launch_aborted(b, s_abort))) break;
@@ -638,16 +641,16 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             const int nt = __shfl_sync(kAll, it.ok ? it.nt : 0, 0);
             const int ft = __shfl_sync(kAll, min(kFoldTiles, it.f->flush_tiles), 0);
             for (int t = 0; t < nt && go; t += ft, ++fb) {
-                const unsigned buf = fb & 1, use = (fb >> 1) & 1;
-                if (buf != mine) continue;
-                // the accumulator's last run has been read (the first two waits pass at once)
-                go = __all_sync(kAll, field_wait(&accempty[buf], use ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE);
+                if ((fb & 1) != mine) continue;
+                const unsigned buf = fb % L::ACCS, use = (fb >> 1) & 1;
+                // the accumulator's last run has been read (the first waits pass at once)
+                go = __all_sync(kAll, field_wait(&accempty[buf], ((fb / L::ACCS) & 1) ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE);
                 if (!go) break;
                 tc_fence_after();
                 const uint32_t d = tmem + buf * L::DCOLS;
-                const uint64_t ab = ah0 + buf * (kFoldTiles * (L::STAGE >> 4));
-                uint64_t* fullb = full + buf * kFoldTiles;
-                uint64_t* emptyb = empty + buf * kFoldTiles;
+                const uint64_t ab = ah0 + mine * (kFoldTiles * (L::STAGE >> 4));
+                uint64_t* fullb = full + mine * kFoldTiles;
+                uint64_t* emptyb = empty + mine * kFoldTiles;
                 const int cnt = min(ft, nt - t);
                 bool ready = mbar_test(&fullb[0], use);
 #pragma unroll
