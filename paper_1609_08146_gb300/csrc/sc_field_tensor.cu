@@ -36,9 +36,9 @@
 //
 // What bounds it.  256 omegas, 512^2 nodes, 4160 points: 52.2 ms, 5.3e12
 // evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
-// The schedulers issue in two thirds of the cycles and shared memory is busy about
-// as long (operand stores, and the MMAs' reads of them); the tensor pipe works a
-// third of the time.  At a few dozen omegas a tile's fixed work (the pair's
+// Shared memory is busy 91% of the time (53% by the LSU, mostly the operands'
+// stores, 38% by the MMAs' reads of them); the schedulers issue in 64% of the
+// cycles, and the tensor pipe works 31%.  At a few dozen omegas a tile's fixed work (the pair's
 // geometry, three rotations, barriers) counts for most of it: at 32 omegas shared
 // memory is busy 80%, the schedulers issue in 69% of the cycles, and the producers
 // wait for a stage a fifth of their time.  No one of them binds alone there:
