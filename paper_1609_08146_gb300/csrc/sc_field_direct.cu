@@ -213,7 +213,11 @@ __global__ void __launch_bounds__(direct_threads(NB, GP), direct_min_blocks(NB, 
                         const int q = g + h * GP;
                         float co[10];
                         const float phi = pair_coefs(nb, j0 + q, P, co);
-                        const float2 rot = phasor_2wphi(d1h, d1l, phi);
+                        // up to 5 omegas a thread the rotation's cost shows: 8 omegas
+                        // 2.82 -> 2.73 ms, 10 3.36 -> 3.22, 20 5.68 -> 5.63 (256^2
+                        // nodes, 4160 points) against sincospif; with more, or one
+                        // thread a point, 0 to 2% slower (registers)
+                        const float2 rot = NB <= 5 ? rotation_2wphi(d1h, d1l, phi) : phasor_2wphi(d1h, d1l, phi);
                         float4* r4 = reinterpret_cast<float4*>(prow + q * ROW);
                         r4[0] = make_float4(co[0], co[1], co[2], co[3]);
                         r4[1] = make_float4(co[4], co[5], co[6], co[7]);
