@@ -114,6 +114,10 @@ __device__ __forceinline__ float2 load_f32(const double2* F, size_t i)
 // (FP64 latency), the others scan 32 values (columns) for their largest entry
 // (memory latency), a power of two of which scales them into [2^11, 2^12); 0 marks
 // a value with an infinity or a NaN.  One launch, so that either hides the other.
+// The exponent spans -116 (entries from 2^127) to 126, the largest whose inverse
+// is normal: entries below 2^-115, subnormal ones among them, come out smaller than
+// 2^11, but all their bits still fit the two halves, whose last place is 2^-24 at
+// most (an entry of 2^-149 scales to 2^-23).
 constexpr int kScanCols = 32;
 
 template <typename T>
@@ -141,8 +145,8 @@ __global__ void __launch_bounds__(kIM) idft_prep_kernel(const __grid_constant__ 
 #pragma unroll
     for (int i = 1; i < kIM / kScanCols; ++i) mx = max(mx, part[i][c]);
     const float f = __int_as_float(mx);
-    const int e = f > 0.f && f < INFINITY ? 11 - ilogbf(f) : 0;  // (an exponent that leaves the scale normal)
-    p.col_scale[field * p.n_vals + v] = mx >= 0x7f800000 ? 0.f : ldexpf(1.f, max(-100, min(100, e)));
+    const int e = f > 0.f && f < INFINITY ? min(11 - ilogbf(f), 126) : 0;
+    p.col_scale[field * p.n_vals + v] = mx >= 0x7f800000 ? 0.f : ldexpf(1.f, e);
 }
 
 template <typename T, int MT>
@@ -239,13 +243,13 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
                 const float sc = c < nv ? scale[c] : 1.f;
                 plain[j] = __ballot_sync(0xffffffffu, sc == 0.f);
                 if (c >= nv || sc == 0.f) continue;
-                const float f = p.scale / sc;
+                const float inv = 1.f / sc;  // (2 dk follows by itself: 2 dk / sc could leave the normal range)
                 float* o = out + (size_t)mw * p.n_vals + v0 + c;
 #pragma unroll
                 for (int r0 = 0; r0 < 32; r0 += 16) {
                     float v[16];
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) v[r] = f * tile[(r0 + r) * (kIV + 1) + c];
+                    for (int r = 0; r < 16; ++r) v[r] = p.scale * (inv * tile[(r0 + r) * (kIV + 1) + c]);
                     if (p.accumulate)
 #pragma unroll
                         for (int r = 0; r < 16; ++r)
