@@ -86,20 +86,25 @@ __device__ __forceinline__ uint64_t global_ns()
 // from working ones.
 enum : int { WAIT_ABORTED = -1, WAIT_EXPIRED = 0, WAIT_DONE = 1 };
 
+__device__ __forceinline__ uint32_t mbar_try(uint32_t addr, unsigned parity)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(addr), "r"(parity), "n"(kSuspendNs)
+        : "memory");
+    return done;
+}
+
 __device__ __forceinline__ int mbar_wait(uint64_t* bar, unsigned parity, const volatile int* abort = nullptr)
 {
     const uint32_t addr = smem_u32(bar);
     uint64_t t0 = 0;
     for (unsigned it = 0; it < kSpinLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(addr), "r"(parity), "n"(kSuspendNs)
-            : "memory");
-        if (done) return WAIT_DONE;
+        if (mbar_try(addr, parity)) return WAIT_DONE;
         if (abort && *abort) return WAIT_ABORTED;
         if ((it & 63) == 0) {
             const uint64_t now = global_ns();

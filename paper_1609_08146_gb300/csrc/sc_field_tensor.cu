@@ -399,7 +399,7 @@ struct ProdSync {
     {
         __syncwarp();
         if (lane == 0) mbar_arrive(bar);
-        return field_wait(bar, phase++ & 1, s_abort, launch_abort, timed_out) == WAIT_DONE;
+        return warp_wait(bar, phase++ & 1, s_abort, launch_abort, timed_out);
     }
 };
 
@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         long long fb = 0;
         bool stop = false;
         for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
-            if (*s_abort) break;
+            if (warp_aborted(s_abort)) break;
             const TItem it = tensor_item(b, item);
             if (!it.ok) continue;
             const int ft = min(kFoldTiles, it.f->flush_tiles);
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             const float2 neg = make_float2(-1.f, -1.f);
             for (int t = 0; t < it.nt; t += ft, ++fb) {
                 const int buf = (int)(fb % L::ACCS);
-                if (field_wait(&accfull[buf], (unsigned)((fb / L::ACCS) & 1), s_abort, b.abort, timed_out) != WAIT_DONE) {
+                if (!warp_wait(&accfull[buf], (unsigned)((fb / L::ACCS) & 1), s_abort, b.abort, timed_out)) {
                     stop = true;
                     break;
                 }
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 if ((fb & 1) != mine) continue;
                 const unsigned buf = fb % L::ACCS, use = (fb >> 1) & 1;
                 // the accumulator's last run has been read (the first waits pass at once)
-                go = __all_sync(kAll, field_wait(&accempty[buf], ((fb / L::ACCS) & 1) ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE);
+                go = warp_wait(&accempty[buf], ((fb / L::ACCS) & 1) ^ 1, s_abort, b.abort, timed_out);
                 if (!go) break;
                 tc_fence_after();
                 const uint32_t d = tmem + buf * L::DCOLS;
@@ -624,8 +624,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
 #pragma unroll
                 for (int i = 0; i < kFoldTiles; ++i) {
                     if (!__all_sync(kAll, ready))
-                        go = __all_sync(kAll,
-                                        field_wait(&fullb[i], use, s_abort, b.abort, timed_out) == WAIT_DONE);
+                        go = warp_wait(&fullb[i], use, s_abort, b.abort, timed_out);
                     if (!go) break;
                     if (i + 1 < kFoldTiles) ready = mbar_test(&fullb[i + 1], use);  // asked for ahead
                     const uint64_t ah = ab + i * (L::STAGE >> 4);
@@ -655,7 +654,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         unsigned fb0 = 0;     // runs of this CTA's items so far
         bool stop = false, plain = false;
         for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
-            if (*s_abort) break;
+            if (warp_aborted(s_abort)) break;
             const TItem it = tensor_item(b, item);
             if (!it.ok) {
                 plain = true;
@@ -684,7 +683,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 // the MMAs have read the stage's last contents (the first use passes at once)
                 const unsigned use = ((fb0 + r) >> 1) & 1;
                 auto stage_free = [&] {
-                    return field_wait(&empty[w], use ^ 1, s_abort, b.abort, timed_out) == WAIT_DONE;
+                    return warp_wait(&empty[w], use ^ 1, s_abort, b.abort, timed_out);
                 };
                 if (!(tr >= 0 ? produce_tile<N2, R>(smem + w * L::STAGE, cur, it, lane, nseg, steps, stage_free)
                               : stage_free())) {
@@ -705,11 +704,11 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             // the MMAs may still read the stage this warp borrows: its last run was
             // the newest one on its half
             const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
-            if (fb0 > half && field_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out) != WAIT_DONE)
+            if (fb0 > half && !warp_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out))
                 stop = true;
             ProdSync ps{psync, s_abort, b.abort, 0, false};
             for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
-                if (*s_abort) break;
+                if (warp_aborted(s_abort)) break;
                 const TItem it = tensor_item(b, item);
                 if (!it.ok && !plain_item<N2, R>(smem, it, w, lane, ps)) break;
             }

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
         unsigned use = 0;
         bool ok = true;
         for (int s0 = 0; s0 < n_stages; s0 += kRunStages, use ^= 1) {
-            ok = field_wait(accfull, use, s_abort, nullptr, timed_out) == WAIT_DONE;
+            ok = warp_wait(accfull, use, s_abort, nullptr, timed_out);
             if (!ok) break;
             tc_fence_after();
             // the truncation's expected loss: a last place for a run of two or three
@@ -279,20 +279,19 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
         }
     } else if (warp == 8) {
         // ---------------- MMA issue (warp-uniform loop, one elected lane) ----------------
-        constexpr unsigned kAll = 0xffffffffu;
         const uint32_t sb = smem_u32(smem);
         bool go = true;
         unsigned run = 0;
         for (int s0 = 0; s0 < n_stages && go; s0 += kRunStages, ++run) {
-            go = __all_sync(kAll, field_wait(accempty, (run & 1) ^ 1, s_abort, nullptr, timed_out) == WAIT_DONE);
+            go = warp_wait(accempty, (run & 1) ^ 1, s_abort, nullptr, timed_out);
             if (!go) break;
             tc_fence_after();
             const int s1 = min(s0 + kRunStages, n_stages);
             for (int s = s0; s < s1; ++s) {
                 const int st = s % L::STAGES;
                 const unsigned use = (s / L::STAGES) & 1;
-                go = __all_sync(kAll, field_wait(&full[st], use, s_abort, nullptr, timed_out) == WAIT_DONE &&
-                                          field_wait(&tfull[st], use, s_abort, nullptr, timed_out) == WAIT_DONE);
+                go = warp_wait(&full[st], use, s_abort, nullptr, timed_out) &&
+                     warp_wait(&tfull[st], use, s_abort, nullptr, timed_out);
                 if (!go) break;
                 tc_fence_after();
                 if (elect_one()) {
@@ -383,7 +382,7 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
                 const float2 v = load_f32(raw + (s % kAhead) * (kIOm * kIV), i * kIV);
                 f[i] = make_float2(v.x * sc, v.y * sc);
             }
-            if (field_wait(&empty[st], ((s / L::STAGES) & 1) ^ 1, s_abort, nullptr, timed_out) != WAIT_DONE) break;
+            if (!warp_wait(&empty[st], ((s / L::STAGES) & 1) ^ 1, s_abort, nullptr, timed_out)) break;
             unsigned char* b = smem + st * L::STAGE + MT * 2 * kAHalf + c * 16;
 #pragma unroll
             for (int k = 0; k < kIOm / 4; ++k)
@@ -392,6 +391,8 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[st]);
         }
+        // (a stage given up on leaves copies on their way into this shared memory)
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();

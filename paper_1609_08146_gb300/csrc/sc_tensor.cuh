@@ -68,6 +68,38 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity)
     return done != 0;
 }
 
+// A bounded wait of a whole warp, with the limits of mbar_wait().  That answers
+// lane by lane, and in the poll where a wait runs out, or sees the abort word, one
+// lane can get another answer than its neighbour; what follows a wait here are
+// warp-wide instructions (tcgen05.ld, shuffles, __syncwarp), which a warp torn apart
+// would never leave.  So every way out of this loop is a vote.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, unsigned parity, volatile int* s_abort, int* launch_abort,
+                                          bool& timed_out)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const uint32_t addr = smem_u32(bar);
+    uint64_t t0 = 0;
+    for (unsigned it = 0; it < kSpinLimit; ++it) {
+        if (__all_sync(kAll, mbar_try(addr, parity))) return true;
+        if (__any_sync(kAll, *s_abort)) return false;
+        if ((it & 63) == 0) {
+            const uint64_t now = global_ns();
+            if (it == 0) t0 = now;
+            else if (__any_sync(kAll, now - t0 > kWaitNs)) break;
+        }
+    }
+    *s_abort = 1;
+    timed_out = true;
+    if (launch_abort) atomicExch(launch_abort, 1);
+    return false;
+}
+
+// The CTA's abort word, as one answer for the warp.
+__device__ __forceinline__ bool warp_aborted(const volatile int* s_abort)
+{
+    return __any_sync(0xffffffffu, *s_abort != 0);
+}
+
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
