@@ -379,7 +379,9 @@ sc_status sc_eval(sc_ctx* ctx, const sc_mirror_t* mirror, const sc_incident_t* i
  *   times          host, n_t values.
  *   E_t,B_t        host or device, float [n_t][n_points][3]; B_t NULL iff
  *                  B_spec is NULL.
- * Errors: SC_ERR_INVALID, SC_ERR_OOM, SC_ERR_CUDA.
+ * Host outputs synchronize the context stream.  Errors: SC_ERR_INVALID, SC_ERR_OOM,
+ * SC_ERR_CUDA, SC_ERR_TIMEOUT (a bounded device wait ran out; outputs undefined;
+ * with device outputs, which do not synchronize, the next call that does reports it).
  */
 sc_status sc_time_domain(sc_ctx* ctx, sc_precision prec, const void* E_spec, const void* B_spec,
                          const double* omegas, int n_omega, int n_points, const double* times,
@@ -619,7 +621,9 @@ enum {
                                 /* the bulk copy of its node tile `value`, so the   */
                                 /* wait for that tile runs out (no fault, no copy   */
                                 /* in flight); the launch then stops and the call   */
-                                /* reports SC_ERR_TIMEOUT                           */
+                                /* reports SC_ERR_TIMEOUT; in the inverse transform */
+                                /* the first CTA skips stage `value` (16 omegas) of */
+                                /* its phase table                                  */
 };
 sc_status sc_set_option(sc_ctx* ctx, int option, long long value);
 

@@ -889,6 +889,7 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     l.table = (unsigned char*)ctx->phasor.p;
     l.dk_rot = dk_rot;
     l.err = ctx->d_err;
+    l.fail_stage = ctx->fail_tile;
     l.accumulate = accumulate;
     for (int pass = 0; pass < (B_spec && !tensor ? 2 : 1); ++pass) {
         l.F = pass == 0 ? dEs : dBs;
@@ -904,7 +905,8 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     if (!out_dev) {
         SC_CUDA(cudaMemcpyAsync(E_t, dEt, out_bytes, cudaMemcpyDeviceToHost, ctx->stream), "download E(t)");
         if (B_t) SC_CUDA(cudaMemcpyAsync(B_t, dBt, out_bytes, cudaMemcpyDeviceToHost, ctx->stream), "download B(t)");
-        SC_CUDA(cudaStreamSynchronize(ctx->stream), "stream synchronize");
+        // (the tensor kernel leaves its outputs unwritten when a wait runs out)
+        return check_device_error(ctx);
     }
     return SC_OK;
 }

@@ -323,12 +323,15 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
         // ---------------- the phase table's stages ----------------
         if (lane == 0) {
             const unsigned char* tab = p.table + (size_t)blockIdx.y * MT * n_stages * 2 * kAHalf;
+            const bool first = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
+            auto lost = [&](int s) { return first && s == p.fail_stage; };
             int issued = 0;
             for (int s = 0; s < n_stages; ++s) {
                 const int st = s % L::STAGES;
                 if (field_wait(&empty[st], ((s / L::STAGES) & 1) ^ 1, s_abort, nullptr, timed_out) != WAIT_DONE) break;
                 // times past the table's last block of 128 have no stage: nothing reads their rows
                 const int blocks = min(MT, p.m_blocks - (int)blockIdx.y * MT);
+                if (lost(s)) continue;
                 mbar_expect_tx(&tfull[st], blocks * 2 * kAHalf);
                 for (int mt = 0; mt < blocks; ++mt)
                     bulk_g2s(smem + st * L::STAGE + mt * 2 * kAHalf, tab + ((size_t)mt * n_stages + s) * 2 * kAHalf,
@@ -338,7 +341,7 @@ __global__ void __launch_bounds__(kIThreads, 1) idft_tensor_kernel(const __grid_
             // no copy may be on its way into this shared memory when the CTA ends:
             // wait (bounded) for the newest copy of every stage
             for (int s = max(0, issued - L::STAGES); s < issued; ++s)
-                if (mbar_wait(&tfull[s % L::STAGES], (s / L::STAGES) & 1) != WAIT_DONE) timed_out = true;
+                if (!lost(s) && mbar_wait(&tfull[s % L::STAGES], (s / L::STAGES) & 1) != WAIT_DONE) timed_out = true;
         }
         __syncwarp();
     } else if (warp >= 12) {

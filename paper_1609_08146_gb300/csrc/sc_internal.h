@@ -204,6 +204,8 @@ struct IdftLaunch {
     double dk_rot = 0.0;    // step of k where the grid is uniform to rounding, else 0
     int* err = nullptr;     // device error word
     int accumulate = 0;     // add to out (a later chunk of omegas) instead of storing
+    int fail_stage = -1;    // failure-path test (tensor kernel): the first CTA leaves the copies
+                            // of this stage of the phase table unissued
     float scale = 0.f;      // 2 dk, and blocks of times (launch_idft_tensor fills them)
     int m_blocks = 0;
 };
