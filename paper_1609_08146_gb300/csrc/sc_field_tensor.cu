@@ -82,12 +82,12 @@ namespace {
 constexpr int kFoldTiles = 5;               // node tiles per run of an accumulator
 constexpr int kStages = 2 * kFoldTiles;     // operand stages (one node tile each): half for either accumulator
 constexpr int kProd = kStages;              // producer warps, each with a stage of its own
-constexpr int kTensorThreads = 512;
+constexpr int kTensorThreads = 512, kWarps = kTensorThreads / 32;
 static_assert(4 + 2 + kProd <= kTensorThreads / 32, "warps");
 // Registers: 128 a thread at launch; the epilogue's warpgroup takes 176 and
 // the other three 112 (128 * 176 + 384 * 112 = 65536).
-constexpr int kEpiRegs = 176, kOtherRegs = 112;
-static_assert(128 * kEpiRegs + 384 * kOtherRegs <= 65536, "register split");
+constexpr int kLaunchRegs = 128, kEpiRegs = 176, kOtherRegs = 112;
+static_assert(128 * kEpiRegs + 384 * kOtherRegs <= 512 * kLaunchRegs, "register split");
 constexpr int kBlkBytes = kTile * 16;           // a block of 8 rows (or columns) of a stage's 32 nodes
 
 // N2 omegas per row phasor, R row phasors (M = 2 R rows of A)
@@ -109,6 +109,9 @@ struct Tens {
     static_assert(2 * NP % 16 == 0, "hi product width");
     static_assert(ACCS * DCOLS <= ALLOC, "tensor memory");
     static_assert(SMEM <= 227 * 1024, "shared memory");
+    // a warp's share of the stages in plain_item(): its sums, or its pair rows
+    static_assert(OFF_BAR / kWarps / 16 * 16 >= R * N2 * kAcc * 4 && OFF_BAR / kWarps / 16 * 16 >= (32 * 16 + 8 * 4) * 4,
+                  "plain loop");
 };
 
 // Stage layout, MN-major: 128 bytes from one block of 8 nodes to the next,
@@ -383,62 +386,94 @@ __device__ __forceinline__ void write_item(const TItem& it, int row, bool own_ro
 }
 
 // ------------------------------------------------------------------------
-// Items whose operands do not fit fp16: the direct kernel's loop on the
-// producer warps.  Warp w sums every eighth node tile for all omegas (lane =
-// 8 consecutive omegas), sharing each tile's pair rows through its stage; every
-// flush the warps' sums are added, in warp order, to the compensated partials.
+// Items whose operands do not fit fp16 (points near the mirror or beyond it): the
+// direct kernel's loop, on all sixteen warps once the tile loop is done and the
+// registers are shared out evenly again.  A warp sums every sixteenth node tile: GP
+// lanes of NB consecutive omegas share a node, 32 / GP nodes side by side, from
+// pair rows in the warp's part of the stages.  Every flush the node groups' sums
+// are added within the warp, then the warps' in warp order to the compensated
+// partials.
+//
+// What bounds it: the FP32 pipe, as in the direct kernel, whose rate it keeps (all
+// points off the focus, 128^2 nodes, 2048 points, this against the direct kernel: 25
+// omegas 1.14 ms and 1.18, 64 2.19 and 2.20, 128 3.99 and 3.92, 256 7.73 and 7.68;
+// ten producer warps with their 112 registers and a seed for every two omegas
+// took 3.33, 3.35, 5.36 and 18.9).  On tables of a few tiles a warp an item's start
+// shows (32^2 nodes, 512 points: 25 omegas 67 us and 133, 128 158 and 142).
 
-// A bounded barrier of the producer warps (false: aborted or expired).
-struct ProdSync {
-    uint64_t* bar;
-    volatile int* s_abort;
-    int* launch_abort;
-    unsigned phase;
-    bool timed_out;
-    __device__ __forceinline__ bool sync(int lane)
-    {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar);
-        return warp_wait(bar, phase++ & 1, s_abort, launch_abort, timed_out);
-    }
-};
-
-template <int N2, int R>
-__device__ __noinline__ bool plain_item(unsigned char* smem, const TItem& it, int w, int lane, ProdSync& ps)
+// lanes per node and omegas per lane, as in the direct kernel's classes from 25 omegas on
+__device__ __forceinline__ int plain_lanes(int n_omega)
 {
-    constexpr int NB = R * N2 / 32;  // omegas per lane
-    using L = Tens<N2, R>;
-    static_assert(L::STAGE >= R * N2 * 12 * 4 && L::STAGE >= 32 * 16 * 4, "stage too small for the plain loop");
-    const FieldLaunch& p = *it.f;
-    float* rows = reinterpret_cast<float*>(smem + w * L::STAGE);
-    const double om0 = (double)p.om_hi0 + (double)p.om_lo0, dom = (double)p.dom_hi + (double)p.dom_lo;
+    return n_omega <= 32 ? 4 : (n_omega <= 64 ? 8 : (n_omega <= 128 ? 16 : 32));
+}
+
+// w + n d as a float-float pair
+__device__ __forceinline__ float2 ff_step(float2 w, float n, float2 d)
+{
+    const float a = n * d.x;
+    float h = w.x, l = fmaf(n, d.x, -a) + fmaf(n, d.y, w.y);
+    two_sum(h, l, a);
+    return make_float2(h, l);
+}
+
+// Halve the slots a lane keeps: lanes that differ in `bit` exchange what the other
+// keeps and add.
+template <int KEEP>
+__device__ __forceinline__ void halve(AccX2* v, int lane, int bit)
+{
+    const bool up = (lane & bit) != 0;
+#pragma unroll
+    for (int j = 0; j < KEEP; ++j)
+#pragma unroll
+        for (int c = 0; c < kAcc / 2; ++c) {
+            const float2 lo = v[j].v[c], hi = v[j + KEEP].v[c];
+            const float2 give = up ? lo : hi, keep = up ? hi : lo;
+            v[j].v[c].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, bit);
+            v[j].v[c].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, bit);
+        }
+}
+
+template <int NB>
+__device__ __forceinline__ void plain_item(unsigned char* smem, int warp_bytes, const FieldLaunch& p, float4 P, int pt,
+                                        int split, int t0, int nt)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gp = plain_lanes(p.n_omega), g = lane & (gp - 1);
+    float* mine = reinterpret_cast<float*>(smem + warp * warp_bytes);
+    float* row0 = mine + (lane & ~(gp - 1)) * 16 + lane / gp * 4;  // the lane's nodes (4 floats of pad: banks)
+    const float2 w = ff_step(make_float2(p.om_hi0, p.om_lo0), (float)(g * NB), make_float2(p.dom_hi, p.dom_lo));
     float kv[NB];
 #pragma unroll
-    for (int j = 0; j < NB; ++j) kv[j] = (float)(6.283185307179586 * (om0 + (double)(lane * NB + j) * dom));
-    const double wg = om0 + (double)(lane * NB) * dom;
-    const float wgh = (float)wg, wgl = (float)(wg - (double)wgh);
-    float2* dst = p.ws + ((size_t)it.split * p.n_pts + it.pt) * (size_t)p.n_omega * kAcc;
-    const int round = max(1, p.flush_tiles) * kProd;  // tiles per flush, all warps
-    for (int r0 = 0; r0 < it.nt || r0 == 0; r0 += round) {
-        AccX2 acc[NB];
+    for (int j = 0; j < NB; ++j) {
+        const float2 k = ff_step(p.steps.k0, (float)(g * NB + j), p.steps.dk);
+        kv[j] = k.x + k.y;
+    }
+    float2* dst = p.ws + ((size_t)split * p.n_pts + pt) * (size_t)p.n_omega * kAcc;
+    const int round = min(max(1, p.flush_tiles), 1 << 20) * kWarps;  // tiles per flush, all warps
+    // fewer tiles than warps (a rim, a small table): `share` warps take a tile's nodes
+    int share = 1;
+    while (2 * share * nt <= kWarps && 2 * share <= gp) share *= 2;
+    const int q0 = warp % share * (gp / share), q1 = q0 + gp / share;
+    for (int r0 = 0; r0 < nt || r0 == 0; r0 += round) {
+        AccX2 acc[8];
 #pragma unroll
-        for (int j = 0; j < NB; ++j)
+        for (int j = 0; j < 8; ++j)
 #pragma unroll
             for (int c = 0; c < kAcc / 2; ++c) acc[j].v[c] = make_float2(0.f, 0.f);
-        for (int t = r0 + w; t < min(it.nt, r0 + round); t += kProd) {
-            const float* nb = p.nodes + (size_t)(it.t0 + t) * kTileFloats;
+        for (int t = r0 + warp / share; t < min(nt, r0 + round); t += kWarps / share) {
+            const float* nb = p.nodes + (size_t)(t0 + t) * kTileFloats;
             float co[10];
-            const float phi = pair_coefs(nb, lane, it.P, co);
+            const float phi = pair_coefs(nb, lane, P, co);
             const float2 rot = phasor_2wphi(p.dom_hi, p.dom_lo, phi);
-            float4* r4 = reinterpret_cast<float4*>(rows + lane * 16);
+            float4* r4 = reinterpret_cast<float4*>(mine + lane * 16 + lane / gp * 4);
             r4[0] = make_float4(co[0], co[1], co[2], co[3]);
             r4[1] = make_float4(co[4], co[5], co[6], co[7]);
             r4[2] = make_float4(co[8], co[9], rot.x, rot.y);
             r4[3] = make_float4(phi, 0.f, 0.f, 0.f);
             __syncwarp();
 #pragma unroll 1
-            for (int q = 0; q < kTile; ++q) {
-                const float4* s4 = reinterpret_cast<const float4*>(rows + q * 16);
+            for (int q = q0; q < q1; ++q) {
+                const float4* s4 = reinterpret_cast<const float4*>(row0 + q * 16);
                 const float4 a0 = s4[0], a1 = s4[1], a2 = s4[2];
                 const float2 cp[10] = {make_float2(a0.x, a0.x), make_float2(a0.y, a0.y), make_float2(a0.z, a0.z),
                                        make_float2(a0.w, a0.w), make_float2(a1.x, a1.x), make_float2(a1.y, a1.y),
@@ -446,10 +481,10 @@ __device__ __noinline__ bool plain_item(unsigned char* smem, const TItem& it, in
                                        make_float2(-a2.y, -a2.y)};
                 const float2 ro = make_float2(a2.z, a2.w);
                 const float2 cc = make_float2(2.f * ro.x, 2.f * ro.x), ncc = make_float2(-cc.x, -cc.x);
-                float2 p0 = phasor_2wphi_mufu(wgh, wgl, s4[3].x);
+                float2 p0 = phasor_2wphi_mufu(w.x, w.y, s4[3].x);
                 float2 p1 = cmul(p0, ro);
                 eval_x2<true>(acc[0], cp, kv[0], p0);
-                if (NB > 1) eval_x2<true>(acc[1], cp, kv[1], p1);
+                eval_x2<true>(acc[1], cp, kv[1], p1);
 #pragma unroll
                 for (int j = 2; j < NB; ++j) {
                     const float2 pn = __ffma2_rn((j & 1) ? cc : ncc, p1, p0);
@@ -460,26 +495,50 @@ __device__ __noinline__ bool plain_item(unsigned char* smem, const TItem& it, in
             }
             __syncwarp();
         }
-        // the warp's sums into its stage, then all warps' sums into the partials
+        // the node groups' sums: every lane ends with 8 gp / 32 of its omegas
+        int slot0 = 0, slots = 8;
+        if (gp <= 16) halve<4>(acc, lane, 16), slots = 4, slot0 += (lane & 16) >> 2;
+        if (gp <= 8) halve<2>(acc, lane, 8), slots = 2, slot0 += (lane & 8) >> 2;
+        if (gp <= 4) halve<1>(acc, lane, 4), slots = 1, slot0 += (lane & 4) >> 2;
 #pragma unroll
-        for (int j = 0; j < NB; ++j)
+        for (int j = 0; j < 8; ++j) {
+            const int slot = slot0 + j;
+            if (j < slots && slot < NB) {
+                const float sg = (slot & 2) ? -1.f : 1.f;  // sign carried by the phasor recurrence
+                float4* r4 = reinterpret_cast<float4*>(mine + (g * NB + slot) * kAcc);
 #pragma unroll
-            for (int c = 0; c < kAcc / 2; ++c) {
-                const float sg = (j & 2) ? -1.f : 1.f;
-                float* r = rows + (lane * NB + j) * kAcc + 2 * c;
-                r[0] = sg * acc[j].v[c].x;
-                r[1] = sg * acc[j].v[c].y;
+                for (int c = 0; c < kAcc / 4; ++c)
+                    r4[c] = make_float4(sg * acc[j].v[2 * c].x, sg * acc[j].v[2 * c].y, sg * acc[j].v[2 * c + 1].x,
+                                        sg * acc[j].v[2 * c + 1].y);
             }
-        if (!ps.sync(lane)) return false;
-        for (int x = w * 32 + lane; x < p.n_omega * kAcc; x += 32 * kProd) {
+        }
+        __syncthreads();
+        for (int x = threadIdx.x; x < p.n_omega * kAcc; x += kTensorThreads) {
             float2 v = r0 == 0 ? make_float2(0.f, 0.f) : dst[x];
-            for (int u = 0; u < kProd; ++u)
-                two_sum(v.x, v.y, reinterpret_cast<const float*>(smem + u * L::STAGE)[x]);
+            for (int u = 0; u < kWarps; ++u) two_sum(v.x, v.y, reinterpret_cast<const float*>(smem + u * warp_bytes)[x]);
             dst[x] = v;
         }
-        if (!ps.sync(lane)) return false;
+        __syncthreads();
     }
-    return true;
+}
+
+// Every item of the CTA that is left to the plain loop.  Inlined at the kernel's end:
+// as a call it slowed the tile loop, whose registers the compiler then divides
+// differently (48 omegas, 256^2 nodes, 4096 points: 7.37 ms, 7.13 inlined).
+__device__ __forceinline__ void plain_items(const BatchLaunch& b, unsigned char* smem, int bytes)
+{
+    const int wb = bytes / kWarps / 16 * 16;
+    for (long long item = blockIdx.x; item < b.n_items; item += gridDim.x) {
+        const TItem it = tensor_item(b, item);
+        if (it.ok) continue;
+        const int lanes = plain_lanes(it.f->n_omega);
+        switch ((it.f->n_omega + lanes - 1) / lanes) {
+        case 5: plain_item<5>(smem, wb, *it.f, it.P, it.pt, it.split, it.t0, it.nt); break;
+        case 6: plain_item<6>(smem, wb, *it.f, it.P, it.pt, it.split, it.t0, it.nt); break;
+        case 7: plain_item<7>(smem, wb, *it.f, it.P, it.pt, it.split, it.t0, it.nt); break;
+        default: plain_item<8>(smem, wb, *it.f, it.P, it.pt, it.split, it.t0, it.nt);
+        }
+    }
 }
 
 // ------------------------------------------------------------------------
@@ -501,9 +560,9 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
     uint64_t* accfull = empty + kStages;                              // [ACCS] accumulator finished
     uint64_t* accempty = accfull + L::ACCS;                           // [ACCS] accumulator read
     uint64_t* drain = accempty + L::ACCS;                             // [2] the MMA warps' last commits
-    uint64_t* psync = drain + 2;                                      // the producer warps among themselves
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(psync + 1);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
     volatile int* s_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* s_plain = s_abort + 1;                              // some item is left to the plain loop
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
@@ -516,8 +575,8 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         }
         mbar_init(&drain[0], 1);
         mbar_init(&drain[1], 1);
-        mbar_init(psync, kProd);
         *s_abort = 0;
+        *s_plain = 0;
         mbar_fence_init();
     }
     if (warp == 4) {
@@ -545,7 +604,10 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
             if (warp_aborted(s_abort)) break;
             const TItem it = tensor_item(b, item);
-            if (!it.ok) continue;
+            if (!it.ok) {
+                *s_plain = 1;
+                continue;
+            }
             const int ft = min(kFoldTiles, it.f->flush_tiles);
             float2 s[L::N / 2], e[L::N / 2];
 #pragma unroll
@@ -652,14 +714,11 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         const unsigned half = w / kFoldTiles;
         const int slot = w % kFoldTiles;
         unsigned fb0 = 0;     // runs of this CTA's items so far
-        bool stop = false, plain = false;
+        bool stop = false;
         for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
             if (warp_aborted(s_abort)) break;
             const TItem it = tensor_item(b, item);
-            if (!it.ok) {
-                plain = true;
-                continue;
-            }
+            if (!it.ok) continue;
             const int nseg = segments(it.f->n_omega, N2);
             const TensorSteps steps = it.f->steps;
             // this warp's stage is number `slot` of every second run; a short run
@@ -696,24 +755,6 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
             }
             fb0 += nruns;
         }
-        // The items left over come last, so that nothing of the loop above lives
-        // across this call: called from there it put 17 loads and 9 stores of local
-        // memory into every tile of 256 omegas (256^2 nodes, 4160 points: 15.98 ms, now
-        // 13.38).
-        if (plain && !stop) {
-            // the MMAs may still read the stage this warp borrows: its last run was
-            // the newest one on its half
-            const unsigned last = fb0 - 1 - ((fb0 - 1 - half) & 1);
-            if (fb0 > half && !warp_wait(&empty[w], (last >> 1) & 1, s_abort, b.abort, timed_out))
-                stop = true;
-            ProdSync ps{psync, s_abort, b.abort, 0, false};
-            for (long long item = blockIdx.x; item < b.n_items && !stop; item += gridDim.x) {
-                if (warp_aborted(s_abort)) break;
-                const TItem it = tensor_item(b, item);
-                if (!it.ok && !plain_item<N2, R>(smem, it, w, lane, ps)) break;
-            }
-            timed_out |= ps.timed_out;
-        }
     }
     if (timed_out) atomicOr(b.err, ERR_TIMEOUT);
     tc_fence_before();
@@ -722,6 +763,12 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(L::ALLOC));
     }
+    // The items left over.  No role runs any more, so the words are the same for
+    // every thread, and the stages are free (the MMAs' last commits have been waited for).
+    if (*s_plain == 0 || *s_abort != 0) return;
+    if (warp < 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kLaunchRegs));
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kLaunchRegs));
+    plain_items(b, smem, L::STAGE * kStages);
 }
 
 float2 ff(double w)
