@@ -379,6 +379,9 @@ sc_status sc_eval(sc_ctx* ctx, const sc_mirror_t* mirror, const sc_incident_t* i
  *   times          host, n_t values.
  *   E_t,B_t        host or device, float [n_t][n_points][3]; B_t NULL iff
  *                  B_spec is NULL.
+ * 16 omegas and more run on the tensor cores where their scratch (8 bytes a value
+ * beside the phase table) fits the context's budget, else on an FP32 kernel, whose
+ * results differ by rounding.
  * Host outputs synchronize the context stream.  Errors: SC_ERR_INVALID, SC_ERR_OOM,
  * SC_ERR_CUDA, SC_ERR_TIMEOUT (a bounded device wait ran out; outputs undefined;
  * with device outputs, which do not synchronize, the next call that does reports it).

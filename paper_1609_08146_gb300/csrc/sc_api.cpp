@@ -48,12 +48,32 @@ sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes)
     return ensure(ctx, b, bytes, ctx->stream);
 }
 
+void give_back_scratch(sc_ctx* ctx, const DevBuf* keep)
+{
+    for (DevBuf* s : {&ctx->phasor})
+        if (s != keep && s->p) {
+            cudaStreamSynchronize(ctx->stream);  // (used on this stream only)
+            cudaFree(s->p);
+            ctx->held -= s->n;
+            *s = DevBuf{};
+        }
+}
+
+bool try_scratch(sc_ctx* ctx, DevBuf& b, size_t bytes)
+{
+    const std::string err = ctx->err;
+    if (ensure(ctx, b, bytes) == SC_OK) return true;
+    ctx->err = err;
+    return false;
+}
+
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes, cudaStream_t sync_stream)
 {
     if (b.n >= bytes) return SC_OK;
     size_t want = std::max(bytes, b.n + b.n / 2);
     if (ctx->budget && ctx->held - b.n + want > ctx->budget) {
         want = bytes;
+        if (ctx->held - b.n + want > ctx->budget) give_back_scratch(ctx, &b);
         if (ctx->held - b.n + want > ctx->budget)
             return fail(ctx, SC_ERR_OOM, "device budget of %zu bytes exceeded (need %zu more)",
                         ctx->budget, want);
@@ -853,9 +873,6 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     const double dk_rot = rotation_step(kv);
     kv.insert(kv.end(), times, times + n_t);  // wavenumbers, then times, one upload
     if ((st = ensure(ctx, ctx->tkval, kv.size() * sizeof(double))) != SC_OK) return st;
-    const bool tensor = sc::idft_on_tensor(n_omega, n_t);
-    if ((st = ensure(ctx, ctx->phasor, tensor ? sc::idft_scratch_bytes(n_omega, n_vals, n_t)
-                                              : (size_t)n_omega * n_t * sizeof(float2))) != SC_OK) return st;
     const void* dEs = E_spec;
     const void* dBs = B_spec;
     if (!in_dev) {
@@ -877,6 +894,11 @@ static sc_status time_domain_unlocked(sc_ctx* ctx, sc_precision prec, const void
     }
     SC_CUDA(cudaMemcpyAsync(ctx->tkval.p, kv.data(), kv.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->stream),
             "upload wavenumbers and times");
+    // the scratch last: where the budget has no room for the tensor kernel's (the FP32
+    // kernel's phase table, padded, and 8 bytes a value), that kernel runs
+    const bool tensor = sc::idft_on_tensor(n_omega, n_t) &&
+                        try_scratch(ctx, ctx->phasor, sc::idft_scratch_bytes(n_omega, n_vals, n_t));
+    if (!tensor && (st = ensure(ctx, ctx->phasor, (size_t)n_omega * n_t * sizeof(float2))) != SC_OK) return st;
     sc::IdftLaunch l;
     l.f64 = prec == SC_FP64;
     l.n_omega = n_omega;

@@ -184,6 +184,12 @@ sc_status cuda_fail(sc_ctx* c, cudaError_t e, const char* what);
 // grow b to at least `bytes` (synchronizing sync_stream before freeing it)
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes, cudaStream_t sync_stream);
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes);
+// Scratch that a call only borrows (no pointer to it outlives the call that asked for
+// it): try_scratch() is ensure() without an error where there is no room, and
+// give_back_scratch() frees what is held of it but `keep`, for an allocation that the
+// budget would refuse otherwise.
+bool try_scratch(sc_ctx* ctx, DevBuf& b, size_t bytes);
+void give_back_scratch(sc_ctx* ctx, const DevBuf* keep);
 bool is_device_ptr(const void* p);
 
 // ---- node tables, spectra and context helpers (sc_tables.cpp)

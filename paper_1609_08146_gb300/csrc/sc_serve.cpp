@@ -243,7 +243,10 @@ void serve(sc_ctx* ctx)
                 // admit only what fits next to every lane's full workspace; the
                 // first request of an idle server is always admitted
                 const bool idle = srv->held == 0 && ids.empty();
-                if (ctx->budget && !idle && ctx->held + srv->held + b + reserve > ctx->budget) break;
+                if (ctx->budget && !idle && ctx->held + srv->held + b + reserve > ctx->budget) {
+                    give_back_scratch(ctx, nullptr);
+                    if (ctx->held + srv->held + b + reserve > ctx->budget) break;
+                }
                 t.bytes = b;
                 srv->held += b;
                 ids.push_back(*it);
