@@ -50,7 +50,7 @@ sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes)
 
 void give_back_scratch(sc_ctx* ctx, const DevBuf* keep)
 {
-    for (DevBuf* s : {&ctx->phasor})
+    for (DevBuf* s : {&ctx->phasor, &ctx->ws64})
         if (s != keep && s->p) {
             cudaStreamSynchronize(ctx->stream);  // (used on this stream only)
             cudaFree(s->p);
@@ -152,7 +152,7 @@ sc_status sc_destroy(sc_ctx* ctx)
     settle_events(ctx);
     for (auto& t : ctx->tables) free_table(ctx, t);
     for (DevBuf* b : {&ctx->pts, &ctx->outE, &ctx->outB, &ctx->tkval, &ctx->phasor,
-                      &ctx->specE, &ctx->specB, &ctx->tE, &ctx->tB, &ctx->fpts, &ctx->fspecE,
+                      &ctx->specE, &ctx->specB, &ctx->tE, &ctx->tB, &ctx->ws64, &ctx->fpts, &ctx->fspecE,
                       &ctx->fspecB, &ctx->ftE, &ctx->ftB, &ctx->mfie_geo, &ctx->mfie_zern, &ctx->mfie_gl,
                       &ctx->mfie_dJ})
         if (b->p) cudaFree(b->p);
@@ -446,12 +446,9 @@ static sc_status eval_unlocked(sc_ctx* ctx, const sc_mirror_t* m, const sc_incid
         }
         a.trig = ctx->d_trig;
         sc::plan_field_f64(a, ctx->device);
-        if (const size_t need = sc::field_f64_workspace(a)) {
-            // a workspace over the budget costs speed, not the call
-            if (ctx->budget && ctx->main.ws.n < need && ctx->held - ctx->main.ws.n + need > ctx->budget) a.n_splits = 1;
-            else if ((st = ensure(ctx, ctx->main.ws, need)) != SC_OK) return st;
-            a.ws = (double*)ctx->main.ws.p;
-        }
+        // (without room for the workspace the sums are the same, in one block's time each)
+        if (const size_t need = sc::field_f64_workspace(a))
+            a.ws = try_scratch(ctx, ctx->ws64, need) ? (double*)ctx->ws64.p : nullptr;
         for (size_t p = 0; p < tab->parts.size(); ++p) {
             const TablePart& tp = tab->parts[p];
             a.surf = tp.d64;

@@ -115,9 +115,10 @@ __device__ __forceinline__ void times_ik(double s[6], double k)
 {
 #pragma unroll
     for (int cc = 0; cc < 3; ++cc) {
+        // (rounded: a sum of several node ranges must not contract the product into its addition)
         const double re = s[2 * cc];
-        s[2 * cc] = -k * s[2 * cc + 1];
-        s[2 * cc + 1] = k * re;
+        s[2 * cc] = __dmul_rn(-k, s[2 * cc + 1]);
+        s[2 * cc + 1] = __dmul_rn(k, re);
     }
 }
 
@@ -247,8 +248,10 @@ __host__ __device__ inline int f64_stride(int gp) { return gp > 1 ? kF64Row + 1 
 // blockIdx.x: points (128 / gp of them), y: omegas (gp NB of them), z: node
 // split.  One split sums surface and rim and writes the outputs; with several,
 // split z < n_splits writes its share's 12 sums to ws and z = n_splits the
-// rim's.
-template <int NB, bool UNI>
+// rim's.  SERIAL: the several splits of a call that has no room for ws, one after
+// another, added and finished in the order of reduce_f64_kernel, so that a result's
+// bits do not depend on the room there was.
+template <int NB, bool UNI, bool SERIAL>
 __global__ void __launch_bounds__(kF64Threads) field_f64_kernel(Field64Launch a)
 {
     extern __shared__ __align__(16) double rows[];
@@ -267,6 +270,27 @@ __global__ void __launch_bounds__(kF64Threads) field_f64_kernel(Field64Launch a)
         ikv[i] = 1.0 / kv[i];
     }
     double sE[NB][6], sB[NB][6];
+    if constexpr (SERIAL) {
+        double tE[NB][6] = {}, tB[NB][6] = {};
+        const int per = (a.n_surf + a.n_splits - 1) / a.n_splits;
+        for (int sp = 0; sp < a.n_splits; ++sp) {
+            const int j0 = min(sp * per, a.n_surf);
+            sum64<NB, UNI>(a, a.surf, j0, min(j0 + per, a.n_surf), x, y, z, g, k0, kv, ikv, rows, stride, sE, sB);
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    tE[i][c] += sE[i][c];
+                    tB[i][c] += sB[i][c];
+                }
+        }
+        sum64<NB, UNI>(a, a.rim, 0, a.n_rim, x, y, z, g, k0, kv, ikv, rows, stride, sE, sB);
+        if (live)
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (n0 + i < a.n_omega) finish64(a, n0 + i, pt, tE[i], tB[i], sE[i], a.accumulate);
+        return;
+    }
     if (a.n_splits > 1) {
         const bool rim = (int)blockIdx.z == a.n_splits;
         const int per = (a.n_surf + a.n_splits - 1) / a.n_splits;
@@ -407,15 +431,16 @@ namespace {
 
 using F64Kernel = void (*)(Field64Launch);
 
+template <bool SERIAL>
 F64Kernel f64_kernel(int nb, bool uni)
 {
     switch (nb) {
-    case 1: return field_f64_kernel<1, false>;
-    case 2: return uni ? field_f64_kernel<2, true> : field_f64_kernel<2, false>;
-    case 3: return uni ? field_f64_kernel<3, true> : field_f64_kernel<3, false>;
-    case 4: return uni ? field_f64_kernel<4, true> : field_f64_kernel<4, false>;
-    case 5: return uni ? field_f64_kernel<5, true> : field_f64_kernel<5, false>;
-    default: return uni ? field_f64_kernel<6, true> : field_f64_kernel<6, false>;
+    case 1: return field_f64_kernel<1, false, SERIAL>;
+    case 2: return uni ? field_f64_kernel<2, true, SERIAL> : field_f64_kernel<2, false, SERIAL>;
+    case 3: return uni ? field_f64_kernel<3, true, SERIAL> : field_f64_kernel<3, false, SERIAL>;
+    case 4: return uni ? field_f64_kernel<4, true, SERIAL> : field_f64_kernel<4, false, SERIAL>;
+    case 5: return uni ? field_f64_kernel<5, true, SERIAL> : field_f64_kernel<5, false, SERIAL>;
+    default: return uni ? field_f64_kernel<6, true, SERIAL> : field_f64_kernel<6, false, SERIAL>;
     }
 }
 
@@ -431,7 +456,7 @@ void plan_field_f64(Field64Launch& a, int device)
     a.nb = a.n_omega >= 6 * a.gp ? 6 : (a.n_omega + a.gp - 1) / a.gp;
     int per_sm = 1, sms = 1;
     const size_t smem = (size_t)kF64Threads * f64_stride(a.gp) * sizeof(double);
-    const F64Kernel kern = f64_kernel(a.nb, a.dk > 0.0);
+    const F64Kernel kern = f64_kernel<false>(a.nb, a.dk > 0.0);
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kF64Threads, smem) != cudaSuccess) per_sm = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) sms = 1;
@@ -462,12 +487,18 @@ int launch_field_f64(const Field64Launch& a, cudaStream_t s)
 {
     const int ppb = kF64Threads / a.gp, opb = a.gp * a.nb;
     const dim3 grid((unsigned)((a.n_pts + ppb - 1) / ppb), (unsigned)((a.n_omega + opb - 1) / opb),
-                    (unsigned)(a.n_splits > 1 ? a.n_splits + 1 : 1));
+                    (unsigned)(a.ws ? a.n_splits + 1 : 1));
     const size_t smem = (size_t)kF64Threads * f64_stride(a.gp) * sizeof(double);
-    f64_kernel(a.nb, a.dk > 0.0)<<<grid, kF64Threads, smem, s>>>(a);  // (plan_field_f64 raised its limit)
-    cudaError_t e = cudaGetLastError();
+    const bool serial = a.n_splits > 1 && !a.ws;
+    const F64Kernel kern = serial ? f64_kernel<true>(a.nb, a.dk > 0.0) : f64_kernel<false>(a.nb, a.dk > 0.0);
+    cudaError_t e = cudaSuccess;
+    if (serial && smem > 48 * 1024)  // (plan_field_f64 raised the other's limit)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return -(int)e;
-    if (a.n_splits <= 1) return 1;
+    kern<<<grid, kF64Threads, smem, s>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return -(int)e;
+    if (!a.ws) return 1;
     const long long total = (long long)a.n_pts * a.n_omega;
     reduce_f64_kernel<<<(unsigned)((total + kF64Red - 1) / kF64Red), 12 * kF64Red, 0, s>>>(a);
     e = cudaGetLastError();

@@ -136,6 +136,7 @@ struct sc_ctx {
     uint64_t tick = 0;
     sch::DevBuf pts, outE, outB, tkval, phasor, specE, specB, tE, tB;
     sch::DevBuf fpts, fspecE, fspecB, ftE, ftB;  // sc_eval_time_domain: points, chunk spectra, E(t), B(t)
+    sch::DevBuf ws64;              // scratch: the FP64 field sum's node splits
     double2* d_trig = nullptr;     // sine and cosine table of the FP64 field sum
     int* d_err = nullptr;
     int* h_err = nullptr;          // pinned

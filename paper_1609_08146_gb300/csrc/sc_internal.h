@@ -174,7 +174,8 @@ struct Field64Launch {
     double2* E; double2* B;              // [n_omega][n_pts][3]
     double dk = 0.0;                     // step of k where the grid is uniform to rounding, else 0
     // plan (plan_field_f64): threads per point, omegas per thread, node splits;
-    // with several splits, ws holds [n_splits + 1][n_omega][n_pts][kAcc] sums
+    // with several splits, ws holds [n_splits + 1][n_omega][n_pts][kAcc] sums, or is
+    // null: then the points' own blocks take the splits one after another
     int gp = 1, nb = 1, n_splits = 1;
     double* ws = nullptr;
     const double2* trig = nullptr;       // kTrigEntries pairs (launch_trig_table)
