@@ -50,8 +50,8 @@ sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes)
 
 void give_back_scratch(sc_ctx* ctx, const DevBuf* keep)
 {
-    for (DevBuf* s : {&ctx->phasor, &ctx->ws64})
-        if (s != keep && s->p) {
+    for (DevBuf* s : {&ctx->phasor, &ctx->ws64, &ctx->main.ws})
+        if (s != keep && s->p && !(s == &ctx->main.ws && ctx->main.ws_in_use)) {
             cudaStreamSynchronize(ctx->stream);  // (used on this stream only)
             cudaFree(s->p);
             ctx->held -= s->n;

@@ -61,6 +61,24 @@ int heuristic_splits(int tiles, long long pb, int slots, double item_evals)
 
 sc_status launch_chunks_direct(sc_ctx* ctx, Lane& ln, std::vector<Chunk>& ch, float2* ws, size_t ws_n);
 
+// What the budget leaves for a lane's workspace beside everything held but scratch
+// (and a launch's descriptors).
+size_t ws_room(const sc_ctx* ctx, const Lane& ln)
+{
+    if (!ctx->budget) return SIZE_MAX;
+    constexpr size_t kDescriptors = 64 << 10;
+    const size_t scratch = ctx->phasor.n + ctx->ws64.n + ctx->main.ws.n + (&ln == &ctx->main ? 0 : ln.ws.n);
+    const size_t others = ctx->held - scratch + kDescriptors;
+    return ctx->budget > others ? ctx->budget - others : 0;
+}
+
+// A lane's workspace while pointers to it are about: no scratch to give back.
+struct WsInUse {
+    Lane& ln;
+    explicit WsInUse(Lane& l) : ln(l) { ln.ws_in_use = true; }
+    ~WsInUse() { ln.ws_in_use = false; }
+};
+
 // Time one chunk with split count S (the chunk's outputs are overwritten later).
 float time_chunk(sc_ctx* ctx, Lane& ln, Chunk c, int S, const Table* tab, float2* ws)
 {
@@ -91,22 +109,31 @@ sc_status choose_splits(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int s
         return SC_OK;
     }
     const auto key = std::make_tuple(c.cls, tiles, tab->n_rim_tiles, c.f.n_pts, c.f.n_omega, c.n_parts);
-    auto hit = ctx->tuned.find(key);
-    if (hit != ctx->tuned.end()) {
-        *S_out = hit->second;
-        return SC_OK;
-    }
     // whole-request workspace of split count s
     auto ws_bytes = [&](int s) {
         const int tps = (tiles + s - 1) / s;
         const int ns = (tiles + tps - 1) / tps;
         return (size_t)(ns + 1) * c.f.n_pts * c.f.n_omega * sc::kAcc * c.n_parts * sizeof(float2);
     };
+    // Splits whose workspace (in point chunks from the cap on) the budget has no room for
+    // are not taken: fewer are slower, but the call runs.  This alone makes the count
+    // depend on what else is held.
+    const size_t room = ws_room(ctx, ln);
+    auto fitting = [&](int s) {
+        while (s > 1 && std::min(ws_bytes(s), ctx->ws_cap) > room) --s;
+        return s;
+    };
+    auto hit = ctx->tuned.find(key);
+    if (hit != ctx->tuned.end()) {
+        *S_out = fitting(hit->second);
+        return SC_OK;
+    }
     int s0 = heuristic_splits(tiles, c.pb, slots, (double)c.ppc * tiles * sc::kTile * c.f.n_omega * c.n_parts);
     // the item-size bound never cuts into points a request that balance alone keeps in one launch
     const int sb = heuristic_splits(tiles, c.pb, slots, 0.0);
     if (ws_bytes(sb) <= ctx->ws_cap)
         while (s0 > sb && ws_bytes(s0) > ctx->ws_cap) --s0;
+    s0 = fitting(s0);
     int best = s0;
     if (ctx->autotune) {
         // candidates around the heuristic, each timed once on the real chunk
@@ -122,7 +149,7 @@ sc_status choose_splits(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int s
             const int tps = (tiles + s - 1) / s;
             const int ns = (tiles + tps - 1) / tps;
             const size_t n = (size_t)(ns + 1) * c.f.n_pts * c.f.n_omega * sc::kAcc * c.n_parts;
-            if (n * sizeof(float2) <= ctx->ws_cap) {
+            if (n * sizeof(float2) <= std::min(ctx->ws_cap, room)) {
                 fit.push_back(s);
                 need = std::max(need, n);
             }
@@ -137,6 +164,7 @@ sc_status choose_splits(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int s
         } else if (fit.size() > 1) {
             sc_status st = ensure(ctx, ln.ws, need * sizeof(float2), ln.stream);
             if (st != SC_OK) return st;
+            const WsInUse use(ln);
             float best_ms = 1e30f;
             for (int s : fit) {
                 const float ms = time_chunk(ctx, ln, c, s, tab, (float2*)ln.ws.p);
@@ -203,6 +231,7 @@ sc_status choose_class(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int* c
         if (t.ws_elems * sizeof(float2) > ctx->ws_cap) continue;  // would need point chunks: not timed
         st = ensure(ctx, ln.ws, t.ws_elems * sizeof(float2), ln.stream);
         if (st != SC_OK) return st;
+        const WsInUse use(ln);
         ms[i] = time_chunk(ctx, ln, t, S, tab, (float2*)ln.ws.p);
     }
     const int best = (ms[1] < 0.99f * ms[0]) ? alt : def;
@@ -633,7 +662,7 @@ double chunk_evals(const Chunk& c)
 // on evaluations) -- and advance i past it.
 sc_status run_chunk_group(sc_ctx* ctx, Lane& ln, std::vector<Chunk>& ch, size_t& i)
 {
-    const size_t cap = std::max<size_t>(ctx->ws_cap / sizeof(float2), 1);
+    const size_t cap = std::max<size_t>(std::min(ctx->ws_cap, ws_room(ctx, ln)) / sizeof(float2), 1);
     const double ecap = ln.max_launch_evals > 0.0 ? ln.max_launch_evals : 1e300;
     size_t j = i, tot = 0;
     double ev = 0.0;
@@ -643,6 +672,7 @@ sc_status run_chunk_group(sc_ctx* ctx, Lane& ln, std::vector<Chunk>& ch, size_t&
     }
     sc_status st = ensure(ctx, ln.ws, tot * sizeof(float2), ln.stream);
     if (st != SC_OK) return st;
+    const WsInUse use(ln);
     std::vector<Chunk> part(ch.begin() + i, ch.begin() + j);
     st = launch_chunks(ctx, ln, part, (float2*)ln.ws.p, tot, ctx->use_graphs && ln.use_graphs);
     if (st != SC_OK) return st;

@@ -113,6 +113,7 @@ struct Lane {
     bool use_graphs = true;         // capture its field launches (if the context does)
     double max_launch_evals = 0.0;  // > 0: bound the evaluations of one launch group
     DevBuf ws, desc, amp, kval;
+    bool ws_in_use = false;         // pointers into ws are about (see give_back_scratch)
     cudaStream_t cap_stream = nullptr;
     std::vector<GraphEntry> graphs;
     // one branch per kernel class of a batch: side streams forked from and
@@ -186,9 +187,9 @@ sc_status cuda_fail(sc_ctx* c, cudaError_t e, const char* what);
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes, cudaStream_t sync_stream);
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes);
 // Scratch that a call only borrows (no pointer to it outlives the call that asked for
-// it): try_scratch() is ensure() without an error where there is no room, and
-// give_back_scratch() frees what is held of it but `keep`, for an allocation that the
-// budget would refuse otherwise.
+// it; the main lane's workspace among it): try_scratch() is ensure() without an error
+// where there is no room, and give_back_scratch() frees what is held of it but `keep`,
+// for an allocation that the budget would refuse otherwise.
 bool try_scratch(sc_ctx* ctx, DevBuf& b, size_t bytes);
 void give_back_scratch(sc_ctx* ctx, const DevBuf* keep);
 bool is_device_ptr(const void* p);

@@ -822,7 +822,6 @@ sc_status get_table(sc_ctx* ctx, const sc_mirror_t* m, const sc_incident_t* in, 
     const size_t b64 = h64.size() * sizeof(sc::Node64);
     t.bytes = b32 + b64;
     // evict least recently used tables while over budget
-    if (ctx->budget && ctx->held + t.bytes > ctx->budget) give_back_scratch(ctx, nullptr);
     while (ctx->budget && ctx->held + t.bytes > ctx->budget && !ctx->tables.empty()) {
         // evict the least recently used table that no call in flight on the host uses
         auto it = ctx->tables.end();
@@ -835,6 +834,7 @@ sc_status get_table(sc_ctx* ctx, const sc_mirror_t* m, const sc_incident_t* in, 
         free_table(ctx, *it);
         ctx->tables.erase(it);
     }
+    if (ctx->budget && ctx->held + t.bytes > ctx->budget) give_back_scratch(ctx, nullptr);
     if (ctx->budget && ctx->held + t.bytes > ctx->budget)
         return fail(ctx, SC_ERR_OOM, "node table of %zu bytes exceeds the device budget", t.bytes);
     cudaError_t e = cudaMalloc(&t.d32, b32);

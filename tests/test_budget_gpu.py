@@ -72,3 +72,71 @@ def test_transform_scratch_is_given_back():
         lo, hi = (lo, mid) if fits(mid, False) else (mid, hi)
     # a kilobyte for the bisection and what a transform keeps beside its scratch (wavenumbers, times)
     assert fits(max(hi + 1024 + 8 * (n_omega + n_t), 8 * (n_omega + n_t) + 8 * n_omega * n_t), True)
+
+
+def _smallest(run, lo=1 << 14, hi=64 << 20):
+    """Smallest budget (to 2 KB) with which run(ctx) is not refused."""
+    def fits(budget):
+        ctx = sc.Context(0, budget_bytes=budget)
+        try:
+            run(ctx)
+            return True
+        except sc.ScError as e:
+            assert e.status == sc.SC_ERR_OOM
+            return False
+        finally:
+            ctx.close()
+
+    while hi - lo > 2048:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid) else (mid, hi)
+    return hi
+
+
+def _request(ctx, n_omega, n_points, n=64):
+    om = np.ones(1) if n_omega == 1 else np.linspace(0.5, 1.5, n_omega)
+    m = ctx.mirror(30.0, 0.0, 60.0, n, n)
+    inc = ctx.incident(profile="gauss", w0=18.0, spectrum=dict(kind="sampled", omega=om, amp=np.ones(n_omega)))
+    return m, inc, om, torch.tensor(np.random.default_rng(n_points).uniform(-1, 1, (n_points, 3)), device="cuda")
+
+
+def _needs(n_omega, n_points, n=64):
+    """Node table (40 and 80 bytes a node, whole tiles, one rim) and the workspace of one split and the rim, and a
+    launch's descriptors, spectrum and slack."""
+    return (n * n + -(-n // 32) * 32) * 120 + 2 * n_points * n_omega * 96 + (80 << 10)
+
+
+@pytest.mark.parametrize("n_omega,n_points", [(1, 1024), (3, 300), (8, 1024), (24, 100), (25, 16), (64, 1024), (256, 100)])
+def test_splits_never_refuse_a_request(n_omega, n_points):
+    """More node splits are faster but need more workspace: a request runs where one split fits, and with room
+    for no more than that its result is that of any other split count to the FP32 path's rounding."""
+    assert _smallest(lambda ctx: ctx.eval(*_request(ctx, n_omega, n_points))) <= _needs(n_omega, n_points)
+    out = []
+    for budget in (0, _needs(n_omega, n_points)):
+        ctx = sc.Context(0, budget_bytes=budget)
+        out.append(ctx.eval(*_request(ctx, n_omega, n_points)))
+        ctx.close()
+    for a, b in zip(*out):
+        # two FP32 sums, each within the path's 1e-5 of the peak
+        assert (a - b).abs().max() <= 2e-5 * b.abs().max()
+
+
+def test_batch_runs_where_its_requests_do():
+    """A batch's launches are cut to what the budget holds."""
+    shapes = [(1 + 7 * i % 50, 40 + 13 * i) for i in range(12)]
+    tables = 12 * _needs(1, 0)
+    largest = max(_needs(*s) - _needs(1, 0) for s in shapes)
+    # (and every request's spectrum and descriptors)
+    assert _smallest(lambda ctx: ctx.eval_batch([_request(ctx, *s) for s in shapes])) <= tables + largest + (64 << 10)
+
+
+def test_workspace_is_given_back():
+    """The workspace that one call leaves does not refuse a call that fits without it."""
+    n_points = 40000
+    pts = np.random.default_rng(1).uniform(-1, 1, (n_points, 3))
+
+    def both(ctx):
+        r = _request(ctx, 8, 1024)
+        ctx.eval(*r)  # the most splits that fit
+        ctx.eval(r[0], r[1], r[2][:1], pts)  # host points and outputs: 24 + 48 bytes a point
+    assert _smallest(both) <= _needs(1, n_points) + 72 * n_points
