@@ -828,7 +828,7 @@ sc_status sc_eval_fp32_static(sc_ctx* ctx, const sc_mirror_t* m, const sc_incide
     f.dom_lo = (float)(domega - (double)f.dom_hi);
     f.ws = ws;
     f.err = ctx->d_err;
-    r = sc::launch_field_f32(f, ctx->stream);
+    r = sc::launch_field_f32(f, tensor_on(ctx), ctx->stream);
     if (r < 0) return cuda_fail(ctx, (cudaError_t)(-r), "field kernel launch");
     ctx->ctr.launches += r;
     ctx->ctr.field_launches += 1;

@@ -430,9 +430,9 @@ int launch_field_batch(int cls, const BatchLaunch& b, int grid, cudaStream_t s)
     }
 }
 
-int launch_field_f32(const FieldLaunch& p, cudaStream_t s)
+int launch_field_f32(const FieldLaunch& p, bool tensor, cudaStream_t s)
 {
-    const int ten = tensor_class(p.n_omega);
+    const int ten = tensor ? tensor_class(p.n_omega) : -1;
     const int cls = ten >= 0 ? ten : field_class(p.n_omega);
     int ppc = 1, slots = 1;
     int dev = 0;

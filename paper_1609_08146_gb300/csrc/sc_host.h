@@ -186,6 +186,8 @@ sc_status cuda_fail(sc_ctx* c, cudaError_t e, const char* what);
 // grow b to at least `bytes` (synchronizing sync_stream before freeing it)
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes, cudaStream_t sync_stream);
 sc_status ensure(sc_ctx* ctx, DevBuf& b, size_t bytes);
+// Whether the options leave the tensor kernel on.
+bool tensor_on(const sc_ctx* ctx);
 // Scratch that a call only borrows (no pointer to it outlives the call that asked for
 // it; the main lane's workspace among it): try_scratch() is ensure() without an error
 // where there is no room, and give_back_scratch() frees what is held of it but `keep`,

@@ -137,8 +137,9 @@ void field_shape(int cls, int device, int* points_per_item, int* resident_ctas);
 int launch_field_batch(int cls, const BatchLaunch& b, int grid, cudaStream_t s);
 
 // Single-request FP32 field sum in grid mode (no device descriptor, no
-// queue).  Returns kernels launched or a negative cudaError_t.
-int launch_field_f32(const FieldLaunch& p, cudaStream_t s);
+// queue), on the tensor kernel where it takes the omega count and `tensor` allows
+// it.  Returns kernels launched or a negative cudaError_t.
+int launch_field_f32(const FieldLaunch& p, bool tensor, cudaStream_t s);
 
 // FP64 cross-split reduction and epilogue: E = a_n (S_E + (i/k_n) S_rim),
 // B = a_n S_B, written as float2 into out[n_omega_total][n_pts_total][3]
