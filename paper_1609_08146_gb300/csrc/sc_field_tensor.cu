@@ -707,7 +707,10 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
         // no MMA may be in flight when the tensor memory is freed
         if (leader) mma_commit(&drain[mine]);
         __syncwarp();
-        if (mbar_wait(&drain[mine], 0) != WAIT_DONE) timed_out = true;
+        if (mbar_wait(&drain[mine], 0) != WAIT_DONE) {
+            timed_out = true;
+            *s_abort = 1;  // (they may still read the stages, which plain_items() would reuse)
+        }
     } else if (prod_index(warp) < kProd) {
         // ---------------- producers ----------------
         const int w = prod_index(warp);  // and its stage
