@@ -95,18 +95,16 @@ template <int N2, int R>
 struct Tens {
     static constexpr int ABYTES = 2 * R / 8 * kBlkBytes;  // one half (hi or lo) of A
     static constexpr int N = 12 * N2;
-    static constexpr int NP = (N + 7) / 8 * 8;     // rounded to core matrices
-    static constexpr int NC = R == 64 ? (NP + 15) / 16 * 16 : NP;  // the lo x hi product (M = 128 wants 16s)
-    static constexpr int DCOLS = NP + NC;          // one accumulator: NP hi hi, then hi lo + lo hi
+    static constexpr int DCOLS = 2 * N;            // one accumulator: hi hi, then hi lo + lo hi
     // Accumulators in tensor memory: with four the MMAs need not wait for the
     // epilogue's last read (25 omegas 6.41 -> 6.23 ms, 64 8.17 -> 7.99); more columns
     // gain nothing at 256 omegas and cost 2% on small tables.
     static constexpr int ACCS = N2 <= 2 ? 4 : 2;
     static constexpr int ALLOC = ACCS * DCOLS <= 64 ? 64 : (ACCS * DCOLS <= 128 ? 128 : (ACCS * DCOLS <= 256 ? 256 : 512));
-    static constexpr int STAGE = 2 * ABYTES + 2 * (NP / 8) * kBlkBytes;
+    static constexpr int STAGE = 2 * ABYTES + 2 * (N / 8) * kBlkBytes;
     static constexpr int OFF_BAR = kStages * STAGE;
     static constexpr int SMEM = OFF_BAR + 256;
-    static_assert(2 * NP % 16 == 0, "hi product width");
+    static_assert(N2 % 2 == 0 && N % (R == 64 ? 16 : 8) == 0, "column pairs, product widths (M = 128 wants 16s)");
     static_assert(ACCS * DCOLS <= ALLOC, "tensor memory");
     static_assert(SMEM <= 227 * 1024, "shared memory");
     // a warp's share of the stages in plain_item(): its sums, or its pair rows
@@ -241,16 +239,15 @@ __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float n
     co[6] = vx * irs; co[7] = vy * irs; co[8] = vz * irs;
     co[9] = co[3] * irs; co[10] = co[4] * irs; co[11] = co[5] * irs;
 
-    // cosines and sines of the column offsets: m steps (odd N2) or m + 1/2 (even)
+    // cosines and sines of the column offsets, m + 1/2 steps
     float trig[N2];
     {
-        float2 q = N2 > 1 ? rotation_2wphi(w.col.x, w.col.y, phi) : make_float2(1.f, 0.f);
-        const float2 full = (N2 & 1) ? q : cmul(q, q);
-        if (N2 & 1) trig[0] = 1.f;
+        float2 q = rotation_2wphi(w.col.x, w.col.y, phi);
+        const float2 full = cmul(q, q);
 #pragma unroll
         for (int m = 0; m < N2 / 2; ++m) {
-            trig[(N2 & 1) + 2 * m] = q.x;
-            trig[(N2 & 1) + 2 * m + 1] = q.y;
+            trig[2 * m] = q.x;
+            trig[2 * m + 1] = q.y;
             if (m + 1 < N2 / 2) q = cmul(q, full);
         }
     }
@@ -262,15 +259,15 @@ __device__ __forceinline__ bool produce_tile(unsigned char* stage, const float n
     if (!wait()) return false;
 
     unsigned char* b_hi = stage + 2 * L::ABYTES + lane * 16;
-    unsigned char* b_lo = b_hi + (L::NP / 8) * kBlkBytes;
+    unsigned char* b_lo = b_hi + (L::N / 8) * kBlkBytes;
 #pragma unroll
-    for (int blk = 0; blk < L::NP / 8; ++blk) {
+    for (int blk = 0; blk < L::N / 8; ++blk) {
         float2 v[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int c0 = blk * 8 + 2 * i;
-            v[i].x = c0 < L::N ? co[c0 % 12] * trig[c0 < L::N ? c0 / 12 : 0] : 0.f;
-            v[i].y = c0 + 1 < L::N ? co[(c0 + 1) % 12] * trig[c0 + 1 < L::N ? (c0 + 1) / 12 : 0] : 0.f;
+            v[i].x = co[c0 % 12] * trig[c0 / 12];
+            v[i].y = co[(c0 + 1) % 12] * trig[(c0 + 1) / 12];
         }
         split_store8(b_hi + blk * kBlkBytes, b_lo + blk * kBlkBytes, v);
     }
@@ -335,17 +332,15 @@ __device__ __forceinline__ void write_item(const TItem& it, int row, bool own_ro
     auto s = [&](int c) { return (c & 1) ? s2[c >> 1].y : s2[c >> 1].x; };
     auto e = [&](int c) { return -((c & 1) ? e2[c >> 1].y : e2[c >> 1].x); };
     float2* base = p.ws + (((size_t)it.split * p.n_pts + it.pt) * (size_t)p.n_omega) * kAcc + (im ? 1 : 0);
-    constexpr int kOff = (N2 + 1) / 2;  // offsets: pairs +-phi, and zero if N2 is odd
 #pragma unroll
-    for (int o = 0; o < kOff; ++o) {
-        const bool zero = (N2 & 1) && o == 0;
-        const int tc = zero ? 0 : ((N2 & 1) ? 2 * o - 1 : 2 * o);  // its cosine column
+    for (int o = 0; o < N2 / 2; ++o) {  // offsets, pairs +-phi
+        const int tc = 2 * o;  // its cosine column
         float2 dst_v[2][6];
         float k_h[2], k_l[2];
         int nn[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {  // h = 0: +phi, 1: -phi
-            const int twice = zero ? 0 : (h == 0 ? 1 : -1) * ((N2 & 1) ? 2 * o : 2 * o + 1);
+            const int twice = (h == 0 ? 1 : -1) * (2 * o + 1);
             nn[h] = n1 * N2 + (twice + N2 - 1) / 2;
             // k_n = k_0 + n dk as a float-float pair, with the sign of ik's product
             const float fn = (float)nn[h], a = fn * p.steps.dk.x;
@@ -357,14 +352,13 @@ __device__ __forceinline__ void write_item(const TItem& it, int row, bool own_ro
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const int c1 = tc * 12 + c, c2 = c1 + 6;
-            // partner's cosine column of S1 and sine (at zero offset: no) column of S2
+            // partner's cosine column of S1 and sine column of S2
             const float p1 = __shfl_xor_sync(0xffffffffu, s(c1), 8), p1e = __shfl_xor_sync(0xffffffffu, e(c1), 8);
-            const float p2 = zero ? 0.f : __shfl_xor_sync(0xffffffffu, s(zero ? c2 : c2 + 12), 8);
-            const float p2e = zero ? 0.f : __shfl_xor_sync(0xffffffffu, e(zero ? c2 : c2 + 12), 8);
-            const float o1 = zero ? 0.f : s(zero ? c1 : c1 + 12), o1e = zero ? 0.f : e(zero ? c1 : c1 + 12);
+            const float p2 = __shfl_xor_sync(0xffffffffu, s(c2 + 12), 8);
+            const float p2e = __shfl_xor_sync(0xffffffffu, e(c2 + 12), 8);
+            const float o1 = s(c1 + 12), o1e = e(c1 + 12);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                if (zero && h == 1) continue;
                 const float q1 = (im ? -1.f : 1.f) * (h == 0 ? 1.f : -1.f);  // S1: cosine rows +-, sine rows -+
                 const float q2 = -q1;                                       // S2: cosine rows -+, sine rows +-
                 float a = p1, al = fmaf(q1, o1e, p1e);
@@ -379,7 +373,7 @@ __device__ __forceinline__ void write_item(const TItem& it, int row, bool own_ro
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (!(zero && h == 1) && own_row && nn[h] < p.n_omega)
+            if (own_row && nn[h] < p.n_omega)
 #pragma unroll
                 for (int c = 0; c < 6; ++c) base[(size_t)nn[h] * kAcc + 2 * c] = dst_v[h][c];
     }
@@ -624,10 +618,10 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                 const float2 unb = make_float2(ub, ub);
                 const uint32_t base = lane_base + buf * L::DCOLS;
 #pragma unroll
-                for (int blk = 0; blk < L::NP / 8; ++blk) {
+                for (int blk = 0; blk < L::N / 8; ++blk) {
                     uint32_t h[8], x[8];
                     tmem_ld8(base + blk * 8, h);
-                    tmem_ld8(base + L::NP + blk * 8, x);
+                    tmem_ld8(base + L::N + blk * 8, x);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -693,10 +687,10 @@ __global__ void __launch_bounds__(kTensorThreads, 1) field_tensor_kernel(const _
                     const uint64_t al = ah + (L::ABYTES >> 4), bh = ah + (2 * L::ABYTES >> 4);
                     if (leader) {
                         if (i < cnt) {
-                            mma_f16(d, ah, bh, mma_idesc(2 * R, 2 * L::NP, true, true), i > 0);            // hi (hi | lo)
-                            mma_f16(d + L::NP, al, bh, mma_idesc(2 * R, L::NC, true, true), 1);            // lo hi
-                            mma_f16(d, ah + 16, bh + 16, mma_idesc(2 * R, 2 * L::NP, true, true), 1);      // nodes 16..31
-                            mma_f16(d + L::NP, al + 16, bh + 16, mma_idesc(2 * R, L::NC, true, true), 1);
+                            mma_f16(d, ah, bh, mma_idesc(2 * R, 2 * L::N, true, true), i > 0);            // hi (hi | lo)
+                            mma_f16(d + L::N, al, bh, mma_idesc(2 * R, L::N, true, true), 1);            // lo hi
+                            mma_f16(d, ah + 16, bh + 16, mma_idesc(2 * R, 2 * L::N, true, true), 1);      // nodes 16..31
+                            mma_f16(d + L::N, al + 16, bh + 16, mma_idesc(2 * R, L::N, true, true), 1);
                         }
                         mma_commit(&emptyb[i]);
                         if (i + 1 == kFoldTiles) mma_commit(&accfull[buf]);
@@ -811,7 +805,7 @@ void tensor_prepare(int cls, FieldLaunch& f)
     f.steps.seed = ff(om0 + (seed_row * n2 + 0.5 * (n2 - 1)) * dom);
     f.steps.row = ff(n2 * dom);
     f.steps.seg = ff(8 * n2 * dom);
-    f.steps.col = ff((n2 & 1) ? dom : 0.5 * dom);
+    f.steps.col = ff(0.5 * dom);
     f.steps.k0 = ff(6.283185307179586 * om0);
     f.steps.dk = ff(6.283185307179586 * dom);
 }
