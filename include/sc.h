@@ -72,7 +72,10 @@ typedef struct sc_incident_t sc_incident_t;
  * Create a context bound to CUDA device `device` and stream `cuda_stream`
  * (a cudaStream_t; NULL = the legacy default stream).  `hbm_budget_bytes`
  * caps the device memory the context itself holds (node tables, workspace,
- * staging); 0 means "no cap beyond what cudaMalloc grants".
+ * staging); 0 means "no cap beyond what cudaMalloc grants".  Workspace that
+ * only makes a call faster is taken where it fits: under a cap that leaves
+ * too little room an FP32 evaluation takes fewer node splits and a transform
+ * the FP32 kernel, whose results differ by rounding (FP64 results do not).
  * Errors: SC_ERR_INVALID (null out, bad device), SC_ERR_CUDA.
  */
 sc_status sc_create(int device, void* cuda_stream, size_t hbm_budget_bytes, sc_ctx** out);

@@ -161,7 +161,9 @@ def load(path: str | None = None):
 
 
 def plan_omega_chunks(n_omega: int, pairs_per_omega: int, ctx=None):
-    """Omega chunk sizes the FP32 path uses for a request (no GPU needed)."""
+    """Omega chunk sizes of a request on the direct and grouped kernels of the
+    FP32 path (no GPU needed).  By default the tensor kernel takes 25 and more
+    omegas, in chunks of up to 256; see sc_plan_omega_chunks in sc.h."""
     lib = load()
     sizes = (ctypes.c_int * (n_omega + 1))()
     n = ctypes.c_int()

@@ -39,9 +39,10 @@ void set_splits(Chunk& c, int S, int tiles)
 }
 
 // Largest work item the split heuristic aims for, in evaluations: about 6 ms
-// of one CTA at the field kernels' rate (2 CTAs per SM).  Serving cuts a long
-// request into launches of a few dozen milliseconds, and such a launch stays
-// balanced only if each CTA takes several items.
+// of one CTA at the direct kernel's rate (2 CTAs per SM), 0.7 ms at the tensor
+// kernel's (one CTA per SM, 256 omegas).  Serving cuts a long request into launches
+// of a few dozen milliseconds, and such a launch stays balanced only if each CTA
+// takes several items.
 constexpr double kMaxItemEvals = 2.5e7;
 
 // items_evals: the evaluations of one item if the chunk had a single split
@@ -187,7 +188,9 @@ bool tensor_on(const sc_ctx* ctx) { return ctx->omega_chunks && ctx->tile_layout
 // autotuner times both on the real chunk, each with its own tuned split
 // count, on the first request of each shape, and keeps the faster unless the
 // default is within 1%.  Chunks above kTuneMaxEvals keep the default.
-// SC_OPT_TILE_LAYOUT 0 / 1 pins the default / the alternative.
+// SC_OPT_TILE_LAYOUT 0 / 1 pins the default / the alternative.  By default the tensor
+// kernel takes 25 to 256 omegas, so that the alternatives of 33 to 128 omegas are
+// timed only where the options turn it off while the autotuner is on.
 sc_status choose_class(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int* cls_out)
 {
     const int def = sc::field_class(c.f.n_omega);
@@ -246,7 +249,9 @@ sc_status choose_class(sc_ctx* ctx, Lane& ln, Chunk& c, const Table* tab, int* c
 // re-measures both tables): every omega count 1..64, and full grouped chunks
 // of 64, 128, ..., 2048 omegas.  A grouped chunk of n > 64 omegas gives every
 // point a power of two threads of 8 omegas, so it takes as long as a full
-// chunk of its capacity (the next power of two >= n).
+// chunk of its capacity (the next power of two >= n).  These are the rates of the
+// direct and grouped kernels: the entries from 25 omegas on and kRateFull plan
+// requests only where the options turn the tensor kernel off.
 constexpr double kRateSmall[65] = {
     0.0,
     3.669, 4.907, 5.611, 6.067, 6.591, 7.171, 6.940, 7.982,  // 1..8

@@ -2,8 +2,8 @@
 // sizes (sc_idft.cu has the tensor-core kernel of the others).
 //
 // field_f64_kernel: the same quadrature of Sec. II Eq. 11 as the FP32 kernel,
-// written the plain way: FP64 throughout, phase R - (z + 2f) + W formed by a
-// direct difference.  It is both a second parity check and the FP64 GPU
+// in FP64 throughout, with the phase R - (z + 2f) + W formed by a direct
+// difference.  It is both a second parity check and the FP64 GPU
 // baseline.  An incident with several node tables runs once per table, the
 // later ones adding to E and B.
 //
@@ -43,7 +43,7 @@ constexpr int kF64Row = 13;  // doubles per shared pair row: ir, phi, U, V, Wv, 
 // sin and cos by table lookup (P. T. P. Tang, "Table-lookup algorithms for
 // elementary functions and their error analysis", 1991): x = j 2 pi / N + r with
 // |r| <= pi / N, the N pairs (cos, sin)(2 pi j / N) from memory and Taylor
-// polynomials of sin r and cos r - 1 (the first terms left out are below 2^-60 for
+// polynomials of sin r and cos r - 1 (the first terms left out are below 2^-59 for
 // N = 1024).  16 FP64 instructions; sincos() takes about 37.  Arguments from 2^30
 // on, infinities and NaN go to sincos().
 constexpr int kTrigN = kTrigEntries;

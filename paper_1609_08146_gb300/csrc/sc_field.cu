@@ -2,7 +2,8 @@
 // kernel and the class dispatch; the direct kernel of requests with few
 // omegas is in sc_field_direct.cu, the tensor-core kernel that takes 25 to 256
 // omegas by default in sc_field_tensor.cu, their shared device helpers in
-// sc_field_common.cuh.
+// sc_field_common.cuh.  With the default options no request reaches the grouped
+// kernel: it serves SC_OPT_OMEGA_CHUNKS = 0, and sc_eval_fp32_static above 256 omegas.
 //
 // Computes, for every observation point r' and frequency omega_n, the
 // quadrature of Sec. II Eq. 11 (physical-optics Stratton-Chu integrals after

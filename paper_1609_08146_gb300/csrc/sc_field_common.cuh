@@ -154,11 +154,12 @@ __device__ __forceinline__ float2 phasor_2wphi(float w_hi, float w_lo, float phi
 }
 
 // The same phasor from the MUFU sine and cosine (__sincosf, absolute error
-// about 4e-7 on [-pi, pi], where the reduced argument pi r lies).  Used only
-// for the direct kernel's seed, whose error is a constant factor on the
-// phasors derived from it: it does not compound along the recurrence, unlike
-// the rotation's, which stays on sincospif.  There the seed is a large share
-// of the per-pair work (the small-omega classes got 2-27% faster).  The
+// about 4e-7 on [-pi, pi], where the reduced argument pi r lies).  Used for the
+// seeds of the direct and the tensor kernel, whose error is a constant factor on
+// the phasors derived from it: it does not compound along the recurrence, unlike
+// the rotation's, which comes from sincospif or rotation_2wphi() below.  In the
+// direct kernel the seed is a large share of the per-pair work (the small-omega
+// classes got 2-27% faster).  The
 // grouped kernel keeps sincospif for its seeds: with a MUFU seed one
 // Laguerre-Gauss configuration of the seeded random tests went from under
 // 5e-6 to 1.005e-5 of the gate metric, for 1.2% of speed.

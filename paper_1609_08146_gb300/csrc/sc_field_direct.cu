@@ -1,7 +1,9 @@
 // sc_field_direct.cu -- the direct FP32 field-sum kernel: chunks of up to
-// 256 omegas (the grouped kernel of sc_field.cu takes larger ones).  The quadrature of Sec. II, Eq. 11 over
-// the node table of the paraboloid (Eq. 21) with the compensated phase of
-// Sec. III.C.1; see sc_field.cu for the summand and the shared structure.
+// 256 omegas (the grouped kernel of sc_field.cu takes larger ones; by default
+// the tensor kernel takes those of 25 to 256, and the layouts for them here run where
+// the options turn it off).  The quadrature of Sec. II, Eq. 11 over the node table of
+// the paraboloid (Eq. 21) with the compensated phase of Sec. III.C.1; see sc_field.cu
+// for the summand and the shared structure.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -34,16 +34,16 @@
 // norms over sizes and beams at random: 1.9e-7 to 4.1e-7 here, 2.8e-7 to
 // 1.1e-6 with the FP32 kernels.
 //
-// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 52.2 ms, 5.3e12
+// What bounds it.  256 omegas, 512^2 nodes, 4160 points: 51.7 ms, 5.4e12
 // evaluations a second (direct kernel, at 0.84 of the FP32 pipe: 232 ms).
-// Shared memory is busy 91% of the time (53% by the LSU, mostly the operands'
+// Shared memory is busy 91% of the time (54% by the LSU, mostly the operands'
 // stores, 38% by the MMAs' reads of them); the schedulers issue in 64% of the
-// cycles, and the tensor pipe works 31%.  At a few dozen omegas a tile's fixed work (the pair's
-// geometry, three rotations, barriers) counts for most of it: at 32 omegas shared
-// memory is busy 80%, the schedulers issue in 69% of the cycles, and the producers
-// wait for a stage a fifth of their time.  No one of them binds alone there:
-// twenty stages (a producer then need not wait) and the halves of A stacked into
-// one M = 128 MMA (fewer MMAs and reads) each gained nothing.
+// cycles, and the tensor pipe works 31%.  At a few dozen omegas a tile's fixed work (the
+// pair's geometry, three rotations, barriers) counts for most of it: at 48 omegas
+// shared memory is busy 75% and the schedulers issue in 68% of the cycles, at 100
+// omegas 86% and 67%.  No one of them binds alone there: twenty stages (a producer
+// then need not wait) and the halves of A stacked into one M = 128 MMA (fewer MMAs
+// and reads) each gained nothing.
 //
 // Where the lines between the classes lie (256^2 nodes, 4160 points, 1e11
 // evaluations a second): 24 omegas, direct 9.8, here 8.5; 25: 8.3 and 10.8; 48:
@@ -65,7 +65,9 @@
 //               are 16 contiguous bytes, so that a warp's stores are
 //               conflict-free); no data passes between lanes.
 // Items are strided over the CTAs (item = blockIdx + i gridDim), which every
-// role follows on its own; all waits are bounded as in the other kernels.
+// role follows on its own; all waits are bounded as in the other kernels, and of a
+// whole warp.  Items whose points do not qualify for fp16 operands come last, on all
+// sixteen warps (plain_items).
 #include <cuda_runtime.h>
 #include <stdint.h>
 

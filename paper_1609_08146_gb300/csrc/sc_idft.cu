@@ -16,10 +16,10 @@
 // What bounds it.  4160 points x 3 components x 256 omegas -> 512 times, E and B:
 // 102 MB in and out (15 us at the copy rate), 13 GFLOP (times three products: 21
 // us at the measured tensor rate).  The FP32 kernel took 2 x 208 us plus the
-// table twice; this one about 78 us and 12 for the table and scales, 436 -> 95 us
-// the call.  What is left is mostly L2: every CTA reads the whole phase table (32
-// KB a stage beside 16 KB of spectra, 460 MB in all at about 5 TB/s); then the
-// stores and the waves' tail (392 CTAs on 152 SMs).
+// table twice; this one about 78 us and 12 for the table and scales, 436 -> 96 us
+// the call.  What is left is mostly L2: every CTA reads its 256 times of the phase
+// table (32 KB a stage beside 16 KB of spectra, 392 x 16 stages: 308 MB in all at
+// about 4 TB/s); then the stores and the waves' tail (392 CTAs on 152 SMs).
 //
 // Structure: a CTA makes 128 values x MT 128 times of one field (16 warps):
 //   warps 0-7   MT sets of four read their 128 times' accumulator (TMEM, all 512

@@ -164,7 +164,8 @@ long long reduce_size(const ReduceLaunch& p);  // its threads
 // by off, total = sum of their reduce_size.
 int launch_reduce_batch(const ReduceLaunch* reqs, int n_req, long long total, cudaStream_t s);
 
-// Plain FP64 path: direct sincos per (point, node, omega).
+// FP64 path (sc_f64_idft.cu): direct phase difference, sines from a table, phases by
+// recurrence on uniform grids.
 struct Field64Launch {
     const Node64* surf; int n_surf;
     const Node64* rim;  int n_rim;

@@ -18,9 +18,9 @@
 // splits in FP64 took four of them (two conversions, two additions) per value
 // and split, one thread per (point, omega) in blocks of 256; now they are paid
 // once per value and table.  Under ncu, cold caches: 1024 points x 1 omega x 64
-// splits 65 -> 11 us (was 4 blocks, serial over the splits: latency), 3001 x 11
-// x 48 splits 176 -> 47 us.  One lane per four splits: with one per sixteen the
-// first took 22 us.
+// splits 230 -> 13 us (was 4 blocks, serial over the splits: latency), 3001 x 11
+// x 48 splits 177 -> 48 us.  One lane per four splits: with one per sixteen the
+// first took twice as long.
 #include <cuda_runtime.h>
 
 #include "sc_internal.h"

@@ -35,6 +35,8 @@ namespace sch {
 // split count is that of the whole request), so results stay bitwise the same
 // as alone.  With SC_OPT_SERVE_PRIORITY = 0 the server uses two lanes of the
 // default priority, first come first served, without bounded launches.
+// (at the rate of the direct kernel, 1.1e12 a second; requests of 25 to 256 omegas run
+// up to five times as fast on the tensor kernel)
 constexpr double kLongEvals = 1e11;        // about 90 ms of field work on one GB300
 constexpr double kGroupEvals = 6e10;       // about 50 ms
 constexpr double kShortBatchEvals = 3e10;
